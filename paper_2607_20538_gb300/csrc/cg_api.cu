@@ -456,7 +456,7 @@ CG_EXPORT int cg_encode(const cg_shape* shape, const cg_params* params, const vo
     a.scales = static_cast<uint32_t*>(out_scales);
     if (tile) {
         bu_maps(shape, z, z.nb * z.pay, z.nb, &a.cmap, &a.smap, true);
-        e = launch_tile_encode_simt(a, st);
+        e = tc_tile_encode_eligible(a) ? tc_launch_tile_encode(a, st) : launch_tile_encode_simt(a, st);
         if (e != cudaSuccess) return cuda_fail(e, "tile encode launch");
         return CG_OK;
     }

@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(kRowThreads) row_encode_kernel(RowArgs a) {
 // Block-uniform tiles: Z = G X for the 16 tokens of a tile, then one min/max range per
 // tile block (16 tokens x blk channels, Sec. 4.3 with T_b = 16 from Sec. 4.2), codes and
 // packing in the per-token row layout, one {scale, zero} pair per tile block.
-// One warp per tile; the CTA shares the (l, s, h) gauge set in shared memory.
+// One warp per tile; the CTA shares the (l, s, h) gauge set in shared memory. Serves the shapes
+// that the tensor-core tile encoder does not take (d other than 128, block < 32, < 64 tokens).
 // ------------------------------------------------------------------------------------
 constexpr int kTileTokens = CG_TILE_TOKENS;
 constexpr int kTileWarpsMax = 16;
