@@ -10,14 +10,12 @@
 //           and is rotated once per query at the end.
 // The token loop reads only codes and scales (no bf16 cache is written or read).
 //
-// A b-bit code q enters the fp32 arithmetic as f = 1 + q 2^-b (bit pattern 0x3F800000 | q << (23-b),
-// two integer operations, exact), so sum_c w_c q_c = 2^b (sum_c w_c f_c - sum_c w_c).
-//
 // Kernels: attn_query_kernel (q' = scale * G_K q); a chunk kernel that writes, per (l, b, h) and
-// part, the part's softmax max, sum and gauge-space weighted value sum (attn_chunk_mma_kernel for
-// 2- and 4-bit codes: many 128-token chunks per CTA, codes staged by bulk copies one chunk ahead,
-// online softmax; attn_chunk_kernel for 3-, 6- and 8-bit codes: one chunk per CTA, all on CUDA
-// cores); attn_combine_kernel (merges the parts, applies G_V^T).
+// part, the part's softmax max (base-2 logarithm), sum and gauge-space weighted value sum:
+// attn_stream_kernel for 2-, 4- and 8-bit codes (both contractions on mma.sync, one warp per token
+// stream), attn_chunk_kernel for 3- and 6-bit codes, whose code pairs straddle words (one
+// 128-token chunk per CTA, all on CUDA cores); attn_combine_kernel (merges the parts, applies
+// G_V^T).
 #include "cg_launch.h"
 #include "cg_sm100.cuh"
 #include "cg_tc_common.cuh"
@@ -43,35 +41,58 @@ __device__ __forceinline__ float code_f(const uint32_t* w, int c) {
 __device__ __forceinline__ float half_lo(uint32_t v) { return h2f_bits(v & 0xffffu); }
 __device__ __forceinline__ float half_hi(uint32_t v) { return h2f_bits(v >> 16); }
 
-constexpr int kQuerySeqs = 4;  // sequences per CTA of the query rotation
+constexpr int kQueries = 8;  // queries per CTA of the query rotation
+constexpr int kQThreads = 256;
+constexpr float kLog2e = 1.4426950408889634f;
 
-// q' = scale * G_K q for the query heads of kQuerySeqs sequences of one (l, h); G_K transposed
-// in shared memory.
-__global__ void __launch_bounds__(kAD) attn_query_kernel(AttnArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int g = a.g;
-    float* Gt = reinterpret_cast<float*>(smem);  // Gt[r][j][i] = G_r[i][j]
-    float* qs = Gt + kAD * g;                    // one query vector
-    const int l = blockIdx.x / a.H, h = blockIdx.x % a.H, c = threadIdx.x;
-    const float* Gsrc = a.G + ((int64_t)(l * 2 + 0) * a.H + h) * (int64_t)kAD * g;
-    for (int e = threadIdx.x; e < kAD * g; e += blockDim.x) {
-        const int r = e / (g * g), rem = e - r * g * g, i = rem / g, j = rem - i * g;
-        Gt[r * g * g + j * g + i] = __ldg(Gsrc + e);
+// q' = scale * G_K q for kQueries queries of one (l, h). The gauge set is staged with rows padded by
+// 16 bytes (coalesced loads, conflict-free 16-byte row reads); a thread owns one output channel and
+// half of the queries, so one gauge value read from shared memory serves four of them.
+__global__ void __launch_bounds__(kQThreads) attn_query_kernel(AttnArgs a) {
+    extern __shared__ __align__(16) float Gs[];  // [128][g + 4], then [kQueries][128] queries
+    const int g = a.g, gp = g + 4;
+    float* qs = Gs + kAD * gp;
+    const int l = blockIdx.x / a.H, h = blockIdx.x - l * a.H;
+    const int n_all = a.B * a.n_rep;  // queries of this (l, h), sequence-major
+    const int q_lo = blockIdx.y * kQueries;
+    const int nq = n_all - q_lo < kQueries ? n_all - q_lo : kQueries;
+    asm volatile("griddepcontrol.launch_dependents;");  // the stream kernel may take free slots and start its copies
+    const float4* Gsrc = reinterpret_cast<const float4*>(a.G + ((int64_t)(l * 2 + 0) * a.H + h) * (int64_t)kAD * g);
+    const int lg = 29 - __clz(g);  // log2(g / 4)
+#pragma unroll 8
+    for (int e = threadIdx.x; e < kAD * g / 4; e += kQThreads)
+        *reinterpret_cast<float4*>(Gs + (e >> lg) * gp + 4 * (e & (g / 4 - 1))) = __ldg(Gsrc + e);
+    const int i = threadIdx.x & (kAD - 1), half = threadIdx.x >> 7;
+    auto row_of = [&](int k) -> int64_t {  // first element of query q_lo + k
+        const int b = (q_lo + k) / a.n_rep, rq = (q_lo + k) - b * a.n_rep;
+        return ((((int64_t)l * a.B + b) * a.H + h) * a.n_rep + rq) * kAD;
+    };
+#pragma unroll
+    for (int k = 0; k < kQueries / 2; k++) {
+        const int q = half * (kQueries / 2) + k;
+        qs[q * kAD + i] = q < nq ? bf16_bits_to_float(a.q[row_of(q) + i]) : 0.0f;
     }
-    const int grp = c / g, i = c - grp * g;
-    const int b_hi = (blockIdx.y + 1) * kQuerySeqs < a.B ? (blockIdx.y + 1) * kQuerySeqs : a.B;
-    for (int b = blockIdx.y * kQuerySeqs; b < b_hi; b++)
-        for (int rq = 0; rq < a.n_rep; rq++) {
-            const int64_t qi = ((((int64_t)l * a.B + b) * a.H + h) * a.n_rep + rq) * kAD;
-            __syncthreads();
-            qs[c] = bf16_bits_to_float(a.q[qi + c]);
-            __syncthreads();
-            const float* Gc = Gt + grp * g * g + i;
-            const float* xq = qs + grp * g;
-            float acc = 0.0f;
-            for (int j = 0; j < g; j++) acc = fmaf(Gc[j * g], xq[j], acc);
-            a.qrot[qi + c] = a.scale * acc;
+    __syncthreads();
+    const float4* row = reinterpret_cast<const float4*>(Gs + i * gp);
+    const float* x0 = qs + half * (kQueries / 2) * kAD + (i & ~(g - 1));
+    float acc[kQueries / 2] = {};
+#pragma unroll 4
+    for (int j = 0; j < g / 4; j++) {
+        const float4 gv = row[j];
+#pragma unroll
+        for (int k = 0; k < kQueries / 2; k++) {
+            const float4 x = *reinterpret_cast<const float4*>(x0 + k * kAD + 4 * j);
+            acc[k] = fmaf(gv.x, x.x, acc[k]);
+            acc[k] = fmaf(gv.y, x.y, acc[k]);
+            acc[k] = fmaf(gv.z, x.z, acc[k]);
+            acc[k] = fmaf(gv.w, x.w, acc[k]);
         }
+    }
+#pragma unroll
+    for (int k = 0; k < kQueries / 2; k++) {
+        const int q = half * (kQueries / 2) + k;
+        if (q < nq) a.qrot[row_of(q) + i] = a.scale * acc[k];
+    }
 }
 
 // Deterministic block reduction of NV values per thread (sum or max) over NT threads, result
@@ -260,485 +281,733 @@ __global__ void __launch_bounds__(kAThreads) attn_chunk_kernel(AttnArgs a) {
         part[r * (kAD + 2) + 2 + c] = kTwoB * (s - Wr[r * 4 + k]) + Zr[r * 4 + k];
     }
     if (tid < NREP) {
-        part[tid * (kAD + 2)] = mx[tid];
+        part[tid * (kAD + 2)] = mx[tid] * kLog2e;
         part[tid * (kAD + 2) + 1] = sm[tid];
     }
 }
 
-// Merge the chunks of one (l, b, h) and apply G_V^T (per gauge group): out fp32.
-__global__ void __launch_bounds__(kAD) attn_combine_kernel(AttnArgs a) {
-    __shared__ float zs[kAD];
-    const int unit = blockIdx.x, c = threadIdx.x;
+constexpr int kCThreads = 512;   // merge: 128 channels x 4 slices of the parts and of the rotation
+constexpr int kCParts = 256;     // parts whose weights are held at a time
+
+// Merges the parts of one (l, b, h) and applies G_V^T (per gauge group): out fp32. It waits for
+// memory, not arithmetic: the parts' maxima, sums and weights are taken one per thread, so that the
+// loop over the parts only loads their value sums, 4 n_rep of a thread in flight; a slice's gauge
+// values are loaded first. 8 units of 57 parts: 17 -> 6 us.
+template <int NREP>
+__global__ void __launch_bounds__(kCThreads) attn_combine_kernel(AttnArgs a) {
+    __shared__ float red[4][NREP][kAD], zs[NREP][kAD], Mw[kCThreads / 32][NREP], Lw[kCThreads / 32][NREP];
+    __shared__ float wgt[kCParts][NREP];
+    const int unit = blockIdx.x, tid = threadIdx.x, c = tid & (kAD - 1), sl = tid >> 7, lane = tid & 31;
     const int l = unit / (a.B * a.H), h = unit % a.H;
     const int g = a.g, grp = c / g, i = c - grp * g;
-    const float* Gv = a.G + ((int64_t)(l * 2 + 1) * a.H + h) * (int64_t)kAD * g + (int64_t)grp * g * g;
-    for (int r = 0; r < a.n_rep; r++) {
-        const float* part = a.part + ((int64_t)unit * a.n_parts * a.n_rep + r) * (kAD + 2);
-        const int64_t stride = (int64_t)a.n_rep * (kAD + 2);
-        float M = -INFINITY;
-        for (int j = 0; j < a.n_parts; j++) M = fmaxf(M, part[j * stride]);
-        float Ls = 0.0f, o = 0.0f;
-        for (int j = 0; j < a.n_parts; j++) {
-            const float e = __expf(part[j * stride] - M);
-            Ls = fmaf(part[j * stride + 1], e, Ls);
-            o = fmaf(part[j * stride + 2 + c], e, o);
-        }
-        __syncthreads();
-        zs[c] = o / Ls;
-        __syncthreads();
-        float acc = 0.0f;
-        for (int j = 0; j < g; j++) acc = fmaf(__ldg(Gv + (int64_t)j * g + i), zs[grp * g + j], acc);
-        a.out[((int64_t)unit * a.n_rep + r) * kAD + c] = acc;
-    }
-}
-
-// ------------------------------------------------------------------------------------
-// Pipelined variant for 2- and 4-bit codes. Scores on tensor cores (mma.sync m16n8k16, bf16 in,
-// fp32 accumulate): a code enters as bf16 2^b + q (exact for b <= 7, three integer operations
-// per pair of codes) and q' as a bf16 hi + lo pair (two MMAs, 2^-16 relative):
-//   D[token][query] = sum_c (2^b + q_tc) q'_c over each 32-channel chunk,
-//   q' . zhat_t = sum_chunks s D + (m - 2^b s) C, C = sum_c q'_c over the chunk.
-// Values on CUDA cores (their contraction runs over tokens, which would need the codes paired
-// along tokens for an MMA): f = 1 + q 2^-b per code, sum_t p_t zhat_tc = 2^b (A - W) + Z with
-// A = sum_t p s_V f, W = sum_t p s_V, Z = sum_t p m_V.
-// ------------------------------------------------------------------------------------
-constexpr int kMThreads = 128;  // 4 warps; each takes 16-token groups in turn
-
-__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%0,%1,%2,%3};\n"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// bf16 pair (low half first) of (2^B + q0, 2^B + q1) from x = q0 | q1 << B (higher bits zero):
-// x * (2^(7-B) + 2^(23-2B)) places q0 at bits 7-B.. and q1 at 23-B.. (the ranges do not overlap),
-// the mask keeps those two fields, and the constant is the bf16 pattern of 2^B twice.
-template <int B>
-__device__ __forceinline__ uint32_t pair_bf16(uint32_t x) {
-    constexpr uint32_t kM = (1u << B) - 1u;
-    constexpr uint32_t kMul = (1u << (7 - B)) | (1u << (23 - 2 * B));
-    constexpr uint32_t kMask = (kM << (7 - B)) | (kM << (23 - B));
-    constexpr uint32_t kOne = ((127u + B) << 7) * 0x10001u;
-    return ((x * kMul) & kMask) | kOne;
-}
-
-// (d0, d1) += a * (b0, b1): one packed fp32 fused multiply-add (each lane rounded once, as fmaf).
-__device__ __forceinline__ void ffma2(float& d0, float& d1, float a, float b0, float b1) {
-    asm("{\n\t.reg .b64 dd, aa, bb;\n\tmov.b64 dd, {%0, %1};\n\tmov.b64 aa, {%2, %2};\n\t"
-        "mov.b64 bb, {%3, %4};\n\tfma.rn.f32x2 dd, aa, bb, dd;\n\tmov.b64 {%0, %1}, dd;\n\t}"
-        : "+f"(d0), "+f"(d1)
-        : "f"(a), "f"(b0), "f"(b1));
-}
-
-// v[i] for a runtime i < 4 without indexing a register array (no local memory).
-template <typename T>
-__device__ __forceinline__ T pick4(const T (&v)[4], int i) {
-    return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3]));
-}
-
-// bf16 hi + lo of two fp32 values, packed as (lo half = first value).
-__device__ __forceinline__ void split2(float v0, float v1, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(v0 - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(v1 - __bfloat162float(h1));
-    hi = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    lo = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-}
-
-// The 2B-bit field of channels (2j, 2j + 1) of a row, j = 4 * wsel + t within word w.
-template <int B>
-__device__ __forceinline__ uint32_t pair_field(uint32_t w, int t) {
-    if (B == 4) return __byte_perm(w, 0u, 0x4440u | (uint32_t)t);
-    return (w >> (4 * t)) & 0xFu;  // B == 2: a pair is one nibble
-}
-
-// Shared-memory layout of attn_chunk_mma_kernel (bytes).
-template <int BITS, int NREP>
-struct MmaSmem {
-    static constexpr int kRow = kAD * BITS / 8;                       // packed token row
-    static constexpr int kStage = kAttnChunk * kRow;                  // one chunk of one tensor
-    static constexpr int bars = 0;                                    // [2 stages][K, V] mbarriers
-    static constexpr int flags = 32;                                  // abort flags
-    static constexpr int codes = 64;                                  // [2 stages][K, V][kStage]
-    static constexpr int qs = codes + 4 * kStage;                     // [NREP][128] q'
-    static constexpr int c32 = qs + NREP * kAD * 4;                   // [NREP][4]
-    static constexpr int run = c32 + NREP * 4 * 4;                    // [NREP] max, sum, alpha; [NREP][4] W, Z
-    static constexpr int scratch = run + NREP * (3 + 8) * 4;          // [4 warps][NREP * 4]
-    static constexpr int outv = scratch + 4 * NREP * 4 * 4;           // [NREP * 4] reduction results
-    static constexpr int sk = outv + NREP * 4 * 4;                    // [2][chunk][4] key scales
-    static constexpr int sv = sk + 2 * kAttnChunk * 4 * 4;            // [2][chunk][4] value scales
-    static constexpr int p = sv + 2 * kAttnChunk * 4 * 4;             // [chunk][NREP] scores / p; red
-    static constexpr int pbytes = NREP * kAttnChunk * 4, rbytes = (kMThreads / 16) * NREP * kAD * 4;
-    static constexpr int total = p + (pbytes > rbytes ? pbytes : rbytes);
-};
-
-// One CTA per (l, b, h) and part: the part's chunks in order, the next chunk's key and value
-// codes arriving by bulk copy into the other stage (and its scales by loads held in registers)
-// while this one is computed, and an online softmax over the chunks (running max; earlier sums
-// rescaled by exp(old - new); each thread keeps its own sums until the end).
-template <int BITS, int NREP>
-__global__ void __launch_bounds__(kMThreads, 3) attn_chunk_mma_kernel(AttnArgs a) {
-    static_assert(BITS == 2 || BITS == 4, "tensor-core attention serves 2- and 4-bit codes");
-    using SL = MmaSmem<BITS, NREP>;
-    constexpr int kWords = kAD * BITS / 32;  // code words per token row
-    constexpr int kRow = SL::kRow;
-    constexpr float kOff = (float)(1 << BITS);
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SL::bars);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::flags);  // [1] stays 0 (drains)
-    float* qs = reinterpret_cast<float*>(smem + SL::qs);
-    float* c32 = reinterpret_cast<float*>(smem + SL::c32);
-    float* Mrun = reinterpret_cast<float*>(smem + SL::run);
-    float* Lrun = Mrun + NREP;
-    float* alpha = Lrun + NREP;
-    float* Wr = alpha + NREP;   // [NREP][4]
-    float* Zr = Wr + NREP * 4;  // [NREP][4]
-    float* scratch = reinterpret_cast<float*>(smem + SL::scratch);
-    uint32_t* SKb = reinterpret_cast<uint32_t*>(smem + SL::sk);
-    uint32_t* SVb = reinterpret_cast<uint32_t*>(smem + SL::sv);
-    float* P = reinterpret_cast<float*>(smem + SL::p);
-    float* outv = reinterpret_cast<float*>(smem + SL::outv);
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    const int unit = blockIdx.y;
-    const int l = unit / (a.B * a.H), bh = unit - l * a.B * a.H, b = bh / a.H, h = bh - (bh / a.H) * a.H;
-    const int blk = a.blk, nb = kAD / blk;
-    const int ch_lo = blockIdx.x * a.chunks_per_part;
-    const int ch_hi = ch_lo + a.chunks_per_part < a.n_chunks ? ch_lo + a.chunks_per_part : a.n_chunks;
-
-    auto chunk_tokens = [&](int ci) -> int {
-        const int64_t c0 = (int64_t)ci * kAttnChunk;
-        return a.T - c0 < kAttnChunk ? (int)(a.T - c0) : kAttnChunk;
-    };
-    auto issue = [&](int ci, int st) {  // thread 0: key and value codes of chunk ci into stage st
-        const uint32_t bytes = (uint32_t)chunk_tokens(ci) * kRow;
-        const int64_t c0 = (int64_t)ci * kAttnChunk;
-        mbar_arrive_expect_tx(&bars[2 * st], bytes);
-        bulk_load(smem + SL::codes + (2 * st) * SL::kStage, a.codes + a.cmap.at(l, 0, b, h, c0), bytes, &bars[2 * st]);
-        mbar_arrive_expect_tx(&bars[2 * st + 1], bytes);
-        bulk_load(smem + SL::codes + (2 * st + 1) * SL::kStage, a.codes + a.cmap.at(l, 1, b, h, c0), bytes,
-                  &bars[2 * st + 1]);
-    };
-
-    // the key and value scales of a chunk's tokens: tokens tid, tid + 128, ... of the chunk
-    auto load_scales = [&](int ci, uint32_t (&ks)[kAttnChunk / kMThreads][4], uint32_t (&vs)[kAttnChunk / kMThreads][4]) {
-        const int64_t c0 = (int64_t)ci * kAttnChunk;
-        const int n = chunk_tokens(ci);
+    constexpr int kStride = NREP * (kAD + 2);
+    const float* part = a.part + (int64_t)unit * a.n_parts * kStride;
+    const int n_parts = (int)(((unit + 1) * a.unit_steps - 1) / a.cta_steps - unit * a.unit_steps / a.cta_steps) + 1;
+    const int per = g / 4;  // g >= 8: gauge rows of this slice
+    const float* Gv = a.G + ((int64_t)(l * 2 + 1) * a.H + h) * (int64_t)kAD * g + (int64_t)grp * g * g + (int64_t)sl * per * g + i;
+    float gv[32];
 #pragma unroll
-        for (int q = 0; q < kAttnChunk / kMThreads; q++) {
-            const int tt = tid + q * kMThreads;
+    for (int j = 0; j < 32; j++) gv[j] = j < per ? __ldg(Gv + (int64_t)j * g) : 0.0f;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the parts
+    float m = -INFINITY;  // thread: query tid mod NREP
+    for (int e = tid; e < n_parts * NREP; e += kCThreads) m = fmaxf(m, part[(int64_t)e * (kAD + 2)]);
 #pragma unroll
-            for (int k = 0; k < 4; k++) ks[q][k] = vs[q][k] = 0u;
-            if (tt < n) {
-                const uint32_t* kp = a.scales + a.smap.at(l, 0, b, h, c0 + tt);
-                const uint32_t* vp = a.scales + a.smap.at(l, 1, b, h, c0 + tt);
-#pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (k < nb) {
-                        ks[q][k] = __ldg(kp + k);
-                        vs[q][k] = __ldg(vp + k);
-                    }
-            }
-        }
-    };
-    auto store_scales = [&](int bufi, const uint32_t (&ks)[kAttnChunk / kMThreads][4],
-                            const uint32_t (&vs)[kAttnChunk / kMThreads][4]) {
-#pragma unroll
-        for (int q = 0; q < kAttnChunk / kMThreads; q++) {
-            const int tt = tid + q * kMThreads;
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                SKb[(bufi * kAttnChunk + tt) * 4 + k] = ks[q][k];
-                SVb[(bufi * kAttnChunk + tt) * 4 + k] = vs[q][k];
-            }
-        }
-    };
-    uint32_t nks[kAttnChunk / kMThreads][4], nvs[kAttnChunk / kMThreads][4];
-
-    if (tid == 0) {
-        abort_flag[0] = 0;
-        abort_flag[1] = 0;
-        for (int k = 0; k < 4; k++) mbar_init(&bars[k], 1);
-        fence_barrier_init();
-    }
-    if (ch_lo < ch_hi) {
-        load_scales(ch_lo, nks, nvs);
-        store_scales(0, nks, nvs);
-    }
-    for (int e = tid; e < NREP * kAD; e += kMThreads) qs[e] = a.qrot[(int64_t)unit * NREP * kAD + e];
-    if (tid < NREP) Mrun[tid] = -INFINITY;
+    for (int off = 16; off >= NREP; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if (lane < NREP) Mw[tid >> 5][lane] = m;
     __syncthreads();
-    if (tid == 0 && ch_lo < ch_hi) issue(ch_lo, 0);
-    if (tid < NREP * 4) {
-        const float* src = qs + (tid >> 2) * kAD + (tid & 3) * 32;
+    m = Mw[0][tid % NREP];
+#pragma unroll
+    for (int w = 1; w < kCThreads / 32; w++) m = fmaxf(m, Mw[w][tid % NREP]);
+    float o[NREP] = {}, ls = 0.0f;
+    for (int j0 = 0; j0 < n_parts; j0 += kCParts) {
+        const int n = n_parts - j0 < kCParts ? n_parts - j0 : kCParts;
+        const float* p0 = part + (int64_t)j0 * kStride;
+        for (int e = tid; e < n * NREP; e += kCThreads) {
+            const float2 ml = *reinterpret_cast<const float2*>(p0 + (int64_t)e * (kAD + 2));
+            const float w = exp2f(ml.x - m);
+            wgt[e / NREP][tid % NREP] = w;
+            ls = fmaf(ml.y, w, ls);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int j = sl; j < n; j += 4)
+#pragma unroll
+            for (int r = 0; r < NREP; r++) o[r] = fmaf(p0[(int64_t)j * kStride + r * (kAD + 2) + 2 + c], wgt[j][r], o[r]);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int off = 16; off >= NREP; off >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, off);
+    if (lane < NREP) Lw[tid >> 5][lane] = ls;
+#pragma unroll
+    for (int r = 0; r < NREP; r++) red[sl][r][c] = o[r];
+    __syncthreads();
+    for (int e = tid; e < NREP * kAD; e += kCThreads) {
+        const int r = e / kAD, k = e % kAD;
         float s = 0.0f;
-        for (int k = 0; k < 32; k++) s += src[k];
-        c32[tid] = s;
+#pragma unroll
+        for (int w = 0; w < kCThreads / 32; w++) s += Lw[w][r];
+        zs[r][k] = ((red[0][r][k] + red[1][r][k]) + (red[2][r][k] + red[3][r][k])) / s;
     }
-    // B fragments of q' (query n = g; rows = channels 16 ks + 2t + {0, 1} and + 8), hi and lo
-    uint32_t qh[8][2], ql[8][2];
-#pragma unroll
-    for (int ks = 0; ks < 8; ks++)
-#pragma unroll
-        for (int hf = 0; hf < 2; hf++) {
-            const int ch = 16 * ks + 8 * hf + 2 * t;
-            const float v0 = g < NREP ? qs[g * kAD + ch] : 0.0f, v1 = g < NREP ? qs[g * kAD + ch + 1] : 0.0f;
-            split2(v0, v1, qh[ks][hf], ql[ks][hf]);
-        }
     __syncthreads();
-
-    // value sums of this thread: channels 8 oct .. 8 oct + 7, tokens vsl, vsl + 8, ...
-    const int oct = tid & 15, vsl = tid >> 4, vbk = (8 * oct) / blk;
-    float acc[NREP][8];
-#pragma unroll
-    for (int r = 0; r < NREP; r++)
-#pragma unroll
-        for (int k = 0; k < 8; k++) acc[r][k] = 0.0f;
-    // this thread's share of the softmax sums: sum p, sum p s_V and sum p m_V per block
-    float lsum[NREP], wsum[NREP][4], zsum[NREP][4];
 #pragma unroll
     for (int r = 0; r < NREP; r++) {
-        lsum[r] = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 4; k++) wsum[r][k] = zsum[r][k] = 0.0f;
-    }
-
-    for (int ci = ch_lo; ci < ch_hi; ci++) {
-        const int it = ci - ch_lo, st = it & 1;
-        const uint32_t par = (uint32_t)(it >> 1) & 1u;
-        const uint32_t* SK = SKb + st * kAttnChunk * 4;
-        const uint32_t* SV = SVb + st * kAttnChunk * 4;
-        if (ci + 1 < ch_hi) load_scales(ci + 1, nks, nvs);  // stored after this chunk
-        const unsigned char* Kc = smem + SL::codes + (2 * st) * SL::kStage;
-        const unsigned char* Vc = Kc + SL::kStage;
-        const int64_t c0 = (int64_t)ci * kAttnChunk;
-        const int n_tok = chunk_tokens(ci);
-        const int ngrp = (n_tok + 15) / 16;
-        // the other stage was released by the barrier that ended the previous chunk
-        if (tid == 0 && ci + 1 < ch_hi) issue(ci + 1, st ^ 1);
-        if (!__syncthreads_and(mbar_wait(&bars[2 * st], par, abort_flag, a.wait_ns))) {
-            if (tid == 0) raise_flag(a.status, CG_FLAG_PIPE_TIMEOUT);
-            // let every copy issued so far land (normal limit): this chunk's stage, and the next
-            // chunk's stage if it was issued
-            for (int sk = 0; sk < 2; sk++) {
-                const int itk = sk == st ? it : it + 1;
-                if (ch_lo + itk >= ch_hi) continue;
-                const uint32_t pk = (uint32_t)(itk >> 1) & 1u;
-                mbar_wait(&bars[2 * sk], pk, abort_flag + 1, tc::kWaitLimitNs);
-                mbar_wait(&bars[2 * sk + 1], pk, abort_flag + 1, tc::kWaitLimitNs);
-            }
-            return;
-        }
-
-        // scores: a warp takes 16 tokens; thread rows g and g + 8, columns (queries) 2t, 2t + 1
-        for (int grp = warp; grp < ngrp; grp += kMThreads / 32) {
-            const int r0 = grp * 16 + g, r1 = r0 + 8;
-            uint32_t w0[kWords], w1[kWords];
-#pragma unroll
-            for (int k = 0; k < kWords; k++) w0[k] = w1[k] = 0u;
-            if (r0 < n_tok) {
-                const uint4* row = reinterpret_cast<const uint4*>(Kc + r0 * kRow);
-#pragma unroll
-                for (int k = 0; k < kWords / 4; k++) {
-                    const uint4 v = row[k];
-                    w0[4 * k] = v.x; w0[4 * k + 1] = v.y; w0[4 * k + 2] = v.z; w0[4 * k + 3] = v.w;
-                }
-            }
-            if (r1 < n_tok) {
-                const uint4* row = reinterpret_cast<const uint4*>(Kc + r1 * kRow);
-#pragma unroll
-                for (int k = 0; k < kWords / 4; k++) {
-                    const uint4 v = row[k];
-                    w1[4 * k] = v.x; w1[4 * k + 1] = v.y; w1[4 * k + 2] = v.z; w1[4 * k + 3] = v.w;
-                }
-            }
-            float d[4][4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) d[k][0] = d[k][1] = d[k][2] = d[k][3] = 0.0f;
-#pragma unroll
-            for (int ks = 0; ks < 8; ks++) {
-                // pair j = 8 ks + t (channels 16 ks + 2t, + 1) and j + 4 (channels + 8)
-                const int wa = BITS == 4 ? 2 * ks : ks, wb = BITS == 4 ? 2 * ks + 1 : ks;
-                const int ta = t, tb = BITS == 4 ? t : t + 4;
-                const uint32_t a0 = pair_bf16<BITS>(pair_field<BITS>(w0[wa], ta));
-                const uint32_t a1 = pair_bf16<BITS>(pair_field<BITS>(w1[wa], ta));
-                const uint32_t a2 = pair_bf16<BITS>(pair_field<BITS>(w0[wb], tb));
-                const uint32_t a3 = pair_bf16<BITS>(pair_field<BITS>(w1[wb], tb));
-                mma16816(d[ks >> 1], a0, a1, a2, a3, qh[ks][0], qh[ks][1]);
-                mma16816(d[ks >> 1], a0, a1, a2, a3, ql[ks][0], ql[ks][1]);
-            }
-#pragma unroll
-            for (int half = 0; half < 2; half++) {
-                const int r = half ? r1 : r0;
-                if (r >= n_tok) continue;
-                uint32_t sz[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) sz[k] = SK[r * 4 + k];
-#pragma unroll
-                for (int cq = 0; cq < 2; cq++) {
-                    const int q = 2 * t + cq;
-                    if (q >= NREP) continue;
-                    float s = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        const uint32_t z = pick4(sz, (32 * k) / blk);
-                        const float sc = half_lo(z), mz = half_hi(z);
-                        s += sc * d[k][2 * half + cq] + (mz - kOff * sc) * c32[q * 4 + k];
-                    }
-                    P[r * NREP + q] = s;
-                }
-            }
-        }
-        __syncthreads();
-
-        // online softmax: the chunk's max, the new running max and the rescale factor
-        {
-            float v[NREP];
-#pragma unroll
-            for (int r = 0; r < NREP; r++) {
-                v[r] = -INFINITY;
-                for (int tt = tid; tt < n_tok; tt += kMThreads) v[r] = fmaxf(v[r], P[tt * NREP + r]);
-            }
-            block_reduce_n<NREP, true, kMThreads>(v, scratch, outv);
-            if (tid < NREP) {
-                const float mn = fmaxf(Mrun[tid], outv[tid]);
-                alpha[tid] = __expf(Mrun[tid] - mn);  // 0 on the first chunk (old max -inf)
-                Mrun[tid] = mn;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int r = 0; r < NREP; r++) {
-                const float al = alpha[r];
-                lsum[r] *= al;
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    wsum[r][k] *= al;
-                    zsum[r][k] *= al;
-                }
-#pragma unroll
-                for (int k = 0; k < 8; k++) acc[r][k] *= al;
-            }
-            for (int tt = tid; tt < n_tok; tt += kMThreads) {
-                uint32_t z[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) z[k] = SV[tt * 4 + k];
-#pragma unroll
-                for (int r = 0; r < NREP; r++) {
-                    const float p = __expf(P[tt * NREP + r] - Mrun[r]);
-                    P[tt * NREP + r] = p;
-                    lsum[r] += p;
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        wsum[r][k] = fmaf(p, half_lo(z[k]), wsum[r][k]);
-                        zsum[r][k] = fmaf(p, half_hi(z[k]), zsum[r][k]);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-
-        // values on CUDA cores: thread = 8 channels (one 32-bit group of 4-bit codes, half of
-        // one for 2-bit) x token slice; sum_t (p s_V) f per channel, f = 1 + q 2^-b
-        if (!__syncthreads_and(mbar_wait(&bars[2 * st + 1], par, abort_flag, a.wait_ns))) {
-            if (tid == 0) raise_flag(a.status, CG_FLAG_PIPE_TIMEOUT);
-            if (ci + 1 < ch_hi) {
-                mbar_wait(&bars[2 * (st ^ 1)], (uint32_t)((it + 1) >> 1) & 1u, abort_flag + 1, tc::kWaitLimitNs);
-                mbar_wait(&bars[2 * (st ^ 1) + 1], (uint32_t)((it + 1) >> 1) & 1u, abort_flag + 1, tc::kWaitLimitNs);
-            }
-            mbar_wait(&bars[2 * st + 1], par, abort_flag + 1, tc::kWaitLimitNs);
-            return;
-        }
-        {
-            const uint32_t* vrow = reinterpret_cast<const uint32_t*>(Vc);
-            for (int tt = vsl; tt < n_tok; tt += kMThreads / 16) {
-                const uint32_t word = vrow[tt * (kRow / 4) + (BITS == 4 ? oct : (oct >> 1))];
-                const uint32_t bits = BITS == 4 ? word : (word >> (16 * (oct & 1)));
-                const float s_v = half_lo(SV[tt * 4 + vbk]);
-                float wgt[NREP];
-#pragma unroll
-                for (int r = 0; r < NREP; r++) wgt[r] = P[tt * NREP + r] * s_v;
-                float f[8];
-#pragma unroll
-                for (int k = 0; k < 8; k++)
-                    f[k] = __uint_as_float(0x3F800000u | (((bits >> (k * BITS)) & ((1u << BITS) - 1u)) << (23 - BITS)));
-#pragma unroll
-                for (int r = 0; r < NREP; r++)
-#pragma unroll
-                    for (int k = 0; k < 8; k += 2) ffma2(acc[r][k], acc[r][k + 1], wgt[r], f[k], f[k + 1]);
-            }
-        }
-        __syncthreads();  // P, the scales and this stage's codes are free for the next chunk
-        if (ci + 1 < ch_hi) store_scales(st ^ 1, nks, nvs);
-    }
-    // the sums over threads (one reduction of each, after the last chunk)
-    block_reduce_n<NREP, false, kMThreads>(lsum, scratch, outv);
-    if (tid < NREP) Lrun[tid] = outv[tid];
-    __syncthreads();
-    {
-        float wv[NREP * 4];
-#pragma unroll
-        for (int r = 0; r < NREP; r++)
-#pragma unroll
-            for (int k = 0; k < 4; k++) wv[r * 4 + k] = wsum[r][k];
-        block_reduce_n<NREP * 4, false, kMThreads>(wv, scratch, outv);
-        if (tid < NREP * 4) Wr[tid] = outv[tid];
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < NREP; r++)
-#pragma unroll
-            for (int k = 0; k < 4; k++) wv[r * 4 + k] = zsum[r][k];
-        block_reduce_n<NREP * 4, false, kMThreads>(wv, scratch, outv);
-        if (tid < NREP * 4) Zr[tid] = outv[tid];
-        __syncthreads();
-    }
-
-    // the slices' sums, then the sum over slices (red reuses P's space)
-    float* red = P;  // [8 slices][NREP][128]
-#pragma unroll
-    for (int r = 0; r < NREP; r++)
-#pragma unroll
-        for (int k = 0; k < 8; k++) red[(vsl * NREP + r) * kAD + 8 * oct + k] = acc[r][k];
-    __syncthreads();
-    float* part = a.part + ((int64_t)unit * a.n_parts + blockIdx.x) * NREP * (kAD + 2);
-    for (int e = tid; e < NREP * kAD; e += kMThreads) {
-        const int r = e / kAD, c = e - r * kAD, k = c / blk;
+        const float* z = zs[r] + grp * g + sl * per;
         float s = 0.0f;
-        for (int q = 0; q < kMThreads / 16; q++) s += red[(q * NREP + r) * kAD + c];
-        part[r * (kAD + 2) + 2 + c] = kOff * (s - Wr[r * 4 + k]) + Zr[r * 4 + k];
+#pragma unroll
+        for (int j = 0; j < 32; j++)
+            if (j < per) s = fmaf(gv[j], z[j], s);
+        red[sl][r][c] = s;
     }
-    if (tid < NREP) {
-        part[tid * (kAD + 2)] = Mrun[tid];
-        part[tid * (kAD + 2) + 1] = Lrun[tid];
+    __syncthreads();
+    for (int e = tid; e < NREP * kAD; e += kCThreads) {
+        const int r = e / kAD, k = e % kAD;
+        a.out[((int64_t)unit * NREP + r) * kAD + k] = (red[0][r][k] + red[1][r][k]) + (red[2][r][k] + red[3][r][k]);
     }
 }
 
-template <int BITS, int NREP>
-size_t mma_smem() {
-    return (size_t)MmaSmem<BITS, NREP>::total;
+// ------------------------------------------------------------------------------------
+// 2-, 4- and 8-bit codes: both contractions on tensor cores (mma.sync m16n8k16, fp16 in, fp32
+// accumulate) straight from the packed words. The codes are the 16-row operand, the queries the
+// 8-column one: up to four queries bring their high parts as columns 0..3 and their low parts as
+// columns 4..7 of the same MMA; eight queries (Q8) take two MMAs. A code enters as the fp16
+// subnormal q 2^(s - 24) (the bits of q in the mantissa, s its offset in the half word), which is
+// exact; the factor 2^s is divided out of the other operand or of the result.
+//   scores  D[token][query] = sum_c q_tc q'_c per quantization block: a register of the code operand
+//           is two channels of one token;
+//           S = sum_blocks s (D + off (C'' - C)) + m C, C = sum_c q'_c over the block.
+//   values  O[channel][query] = sum_t q_tc w_t with w = p s_V: a register of the code operand is one
+//           channel of two tokens (a byte permute per word and half); the weights leave the score
+//           MMA as rows of tokens and become its operand by one 8x8 transpose (movmatrix);
+//           sum_t p m_V is kept per block and added at the end.
+// High + low carry 22 bits (w: of the value, q': of hi + lo). For 2- and 4-bit codes q' is its bf16
+// hi + lo pair (16 bits) and off = 2^b: the same operands, in another form, as (2^b + q) against
+// that pair; for 8-bit codes q' is the fp32 value and off = 0.
+// The MMA accumulators hold one step's tokens only and are added to fp32 sums in registers (rounded
+// to nearest), so the tensor core's own accumulation covers at most 64 tokens.
+// One warp per token stream: it has its own buffers in shared memory, its own online softmax, and
+// meets the other three warps of its CTA only for the queries and at the end of the part. The next
+// step's key codes are copied (bulk) while this step's values are summed, its value codes during
+// the next scores; scales go through registers a step ahead (they have no 16-byte alignment) and
+// are stored as fp32 records that the packed arithmetic over two queries reads directly.
+// Bound by instruction issue and the ALU pipe (about 20 warp instructions a token at 4 bits and two
+// blocks per row, 7.5 of them unpacking; 87 in the kernel it replaced, whose value sums ran on CUDA
+// cores; with the queries as the 16-row operand instead, twice the MMAs for four queries, 308 us
+// against 298). One layer, 64 sequences x 8 heads x 16,384 tokens, 4 bits, 4 queries a head: whole
+// call 1043 -> 281 us (stream kernel 255 us, 4.7 TB/s, 70 % of measured HBM); one 32,767-token
+// sequence at 8 bits 280 -> 43 us.
+// ------------------------------------------------------------------------------------
+constexpr int kSThreads = 128;
+constexpr int kSWarps = kSThreads / 32;
+constexpr int kSCtas = 3;  // per SM: 168 registers a thread; four CTAs (128 registers) spill
+
+template <int BITS, int NB>
+struct StreamCfg {
+    static constexpr int kTok = BITS == 8 ? 32 : 64;           // tokens of a step
+    static constexpr int kRow = kAD * BITS / 8;                // packed token row
+    static constexpr int kCodes = kTok * kRow;                 // one tensor's codes of a step
+    static constexpr int kRecs = kTok * NB;                    // scale records {s, s, m, m} of a step
+    static constexpr int kWarp = 2 * kCodes + 2 * kRecs * 16;  // a warp's K, V codes and K, V scales
+    static constexpr int kBars = 128;                          // mbarriers and flags
+    static constexpr int kQ = 8 * 32 * 16;                     // the score MMAs' query operand
+    static constexpr int kStat = 8 * (2 * NB + 1) * 4;         // per query: C, off (C'' - C), unit
+    static constexpr int kFixed = (kBars + kQ + kStat + 127) / 128 * 128;
+    static constexpr int kTotal = kFixed + kSWarps * kWarp;
+    static constexpr int kPass = NB == 1 ? 2 : NB;             // value passes: 16 / kPass channels each
+    static constexpr int kVC = 16 / kPass;                     // codes per token, lane and pass
+    static_assert(kWarp % 16 == 0 && kCodes % 16 == 0, "aligned parts");
+    static_assert(kWarp >= 8 * (kAD + 2) * 4, "the merge reuses the buffers");
+};
+
+// Codes packed in half words: code i of a half word sits at bit BITS * i. It enters at a bit near the
+// top of the fp16 mantissa (at most bits 2..9): the MMA aligns a subnormal's product by the lowest
+// normal exponent, so a code left in the lowest mantissa bits loses the bits above it (4-bit codes in
+// place: attention 5e-5 off instead of 2e-5, 2-bit ones 1.3e-4). Codes share a shift of the whole
+// word where they can.
+template <int BITS>
+__device__ constexpr int code_shift(int i) {
+    return BITS == 8 ? 2 : (BITS == 4 ? 4 : 6 + 2 * (i & 1));
+}
+template <int BITS>
+__device__ __forceinline__ uint32_t code_pair(uint32_t x, int i) {
+    constexpr uint32_t kM = ((1u << BITS) - 1u) * 0x10001u;
+    const int up = code_shift<BITS>(i) - BITS * i;
+    return (up >= 0 ? x << up : x >> -up) & (kM << code_shift<BITS>(i));
 }
 
-template <int BITS, int NREP>
-cudaError_t launch_mma_chunks(const AttnArgs& a, cudaStream_t st) {
-    const size_t smem = mma_smem<BITS, NREP>();
-    cudaError_t e = cudaFuncSetAttribute(attn_chunk_mma_kernel<BITS, NREP>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Transposes an 8x8 matrix of 16-bit values: lane (g, t) gives row g, columns 2t, 2t + 1 and gets
+// row 2t, 2t + 1 of column g.
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t v) {
+    uint32_t r;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
+}
+
+__device__ __forceinline__ float ex2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+
+// (v0, v1) as fp16 high and low parts, each packed low half first.
+__device__ __forceinline__ void split_f16(float v0, float v1, uint32_t& hi, uint32_t& lo) {
+    const __half2 h = __floats2half2_rn(v0, v1);
+    const float2 f = __half22float2(h);
+    const float2 r = __fadd2_rn(make_float2(v0, v1), make_float2(-f.x, -f.y));
+    const __half2 w = __floats2half2_rn(r.x, r.y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    lo = *reinterpret_cast<const uint32_t*>(&w);
+}
+
+__device__ __forceinline__ float2 scale_zero_of(uint32_t v) {
+    return __half22float2(*reinterpret_cast<const __half2*>(&v));
+}
+
+template <int BITS, int NB, bool Q8>
+__global__ void __launch_bounds__(kSThreads, kSCtas) attn_stream_kernel(AttnArgs a) {
+    static_assert(BITS == 2 || BITS == 4 || BITS == 8, "codes that do not straddle half words");
+    using C = StreamCfg<BITS, NB>;
+    constexpr int kTok = C::kTok, kTiles = kTok / 16, kBlk = kAD / NB;
+    constexpr int kKC = kBlk / 4;                            // key codes per token, lane and block
+    constexpr int kLaneBits = BITS * kKC >= 32 ? 16 : 8;     // key pairs: half words, or bytes of one half word
+    constexpr int kCL = kLaneBits / BITS;                    // codes per half word (byte)
+    constexpr int kKX = kKC / (2 * kCL);                     // words per block
+    constexpr int kKs = kKC / 4;                             // MMA steps per block
+    constexpr int kPass = C::kPass, kVC = C::kVC;
+    constexpr int kVBits = kVC * BITS;                       // value codes per token, lane and pass
+    constexpr int kVL = kVBits >= 16 ? 16 / BITS : kVC;      // codes per half word
+    constexpr int kVX = kVC / kVL;                           // half words
+    constexpr int kItems = C::kRecs / 32;                    // scale records a lane prepares per tensor
+    constexpr float kOff = BITS == 8 ? 0.0f : (float)(1 << BITS);
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem) + 2 * warp;  // this warp's K and V codes
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 64) + 2 * warp;  // [1] stays 0 (drains)
+    uint4* qb = reinterpret_cast<uint4*>(smem + C::kBars) + lane;   // [step][lane]: high b0, b1, low b0, b1
+    float* stat = reinterpret_cast<float*>(smem + C::kBars + C::kQ);  // [query][C, off (C'' - C) per block, unit]
+    unsigned char* kst = smem + C::kFixed + warp * C::kWarp;
+    unsigned char* vst = kst + C::kCodes;
+    float4* sf = reinterpret_cast<float4*>(vst + C::kCodes);  // [K, V][token][block]
+    // row r of an 8-token matrix is token (r >> 1) + 4 (r & 1), so that the tokens a lane's value
+    // operand takes (rows 2t, 2t + 1) are t and t + 4: fewer bank conflicts than neighbours
+    const int tg = (g >> 1) + 4 * (g & 1);
+
+    const int tsh = a.smap.tshift;
+    // scale records of a lane: words lane_off + e_off of a step's rows of NB words, one row per token
+    // or per 16-token tile
+    const int lane_off = tsh ? (NB == 1 ? lane >> 4 : lane % NB) : lane;
+    if (lane == 0) {
+        abort_flag[0] = 0;
+        abort_flag[1] = 0;
+        mbar_init(&bars[0], 1);
+        mbar_init(&bars[1], 1);
+        fence_barrier_init();
+    }
+    __syncwarp();
+    uint32_t phase = 0;  // copies completed by this warp (K and V alike)
+    bool dead = false;   // a wait of this warp ran out
+
+    // this CTA's share of all units' steps: whole segments of one unit each, one part per segment
+    int64_t pos = (int64_t)blockIdx.x * a.cta_steps;
+    const int64_t pos_end = pos + a.cta_steps < a.all_steps ? pos + a.cta_steps : a.all_steps;
+    while (pos < pos_end) {
+    const int unit = (int)(pos / a.unit_steps);
+    const int64_t in_unit = pos - unit * a.unit_steps;
+    const int64_t seg = pos_end - pos < a.unit_steps - in_unit ? pos_end - pos : a.unit_steps - in_unit;
+    const int slot = (int)(blockIdx.x - unit * a.unit_steps / a.cta_steps);
+    pos += seg;
+    const int l = unit / (a.B * a.H), bh = unit - l * a.B * a.H, b = bh / a.H, h = bh - (bh / a.H) * a.H;
+
+    // tokens [lo, hi); a step of the CTA is kSWarps steps of kTok tokens, one per warp
+    const int64_t lo = in_unit * (kSWarps * kTok);
+    const int64_t hi = lo + seg * (kSWarps * kTok) < a.T ? lo + seg * (kSWarps * kTok) : a.T;
+    const int steps_all = (int)((hi - lo + kTok - 1) / kTok);
+    const int steps = steps_all > warp && !dead ? (steps_all - warp + kSWarps - 1) / kSWarps : 0;
+    const uint8_t* kcodes = a.codes + a.cmap.at(l, 0, b, h, lo + warp * kTok);
+    const uint8_t* vcodes = a.codes + a.cmap.at(l, 1, b, h, lo + warp * kTok);
+    const uint32_t* ksc = a.scales + a.smap.at(l, 0, b, h, lo + warp * kTok) + lane_off;
+    const uint32_t* vsc = a.scales + a.smap.at(l, 1, b, h, lo + warp * kTok) + lane_off;
+    const int sc_step = ((kSWarps * kTok) >> tsh) * NB;  // scale words from one step of a warp to its next
+    const int n_part = (int)(hi - lo);  // a part is shorter than 2^31 tokens
+
+    auto step_tokens = [&](int i) -> int {
+        const int left = n_part - (warp + i * kSWarps) * kTok;
+        return left < kTok ? left : kTok;
+    };
+    auto load_codes = [&](int i, int which) {  // lane 0: K (0) or V (1) codes of step i
+        const uint32_t bytes = (uint32_t)step_tokens(i) * C::kRow;
+        mbar_arrive_expect_tx(&bars[which], bytes);
+        bulk_load(which ? vst : kst, (which ? vcodes : kcodes) + (int64_t)i * (kSWarps * C::kCodes), bytes, &bars[which]);
+    };
+    uint32_t nsc[2][kItems];  // scales of a step: record r = (token, block)
+    auto load_scales = [&](int i) {  // called for i = 0, 1, ... in turn
+        const int n = step_tokens(i);
+#pragma unroll
+        for (int e = 0; e < kItems; e++) {
+            const bool ok = n == kTok || (lane + 32 * e) / NB < n;  // tokens that do not exist: zero scale and zero
+            const int at = tsh ? ((32 * e / NB) >> 4) * NB : 32 * e;
+            nsc[0][e] = ok ? __ldg(ksc + at) : 0u;
+            nsc[1][e] = ok ? __ldg(vsc + at) : 0u;
+        }
+        ksc += sc_step;
+        vsc += sc_step;
+    };
+    if (steps > 0) {
+        if (lane == 0) {
+            load_codes(0, 0);
+            load_codes(0, 1);
+        }
+        load_scales(0);
+    }
+
+    // Query operand of the scores: column g, this lane's channels (lane t: codes t * kKC .. of each
+    // block); column g is query g (Q8: high and low operands), or query g & 3, high part for g < 4
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the rotated queries
+    {
+        const int qi = Q8 ? g : g & 3;
+        const float* qrow = a.qrot + ((int64_t)unit * a.n_rep + qi) * kAD;
+        auto value = [&](int ch) { return qi < a.n_rep ? qrow[ch] : 0.0f; };
+        auto rounded = [&](float v) {  // the value the contraction sees
+            if constexpr (BITS == 8) return v;
+            const float hb = __bfloat162float(__float2bfloat16_rn(v));
+            return hb + __bfloat162float(__float2bfloat16_rn(v - hb));
+        };
+        float amax = 0.0f, c1[NB], c2[NB];
+#pragma unroll
+        for (int k = 0; k < NB; k++) {
+            c1[k] = c2[k] = 0.0f;
+#pragma unroll 8
+            for (int j = 0; j < kKC; j++) {
+                const float v = value(k * kBlk + t * kKC + j), r = rounded(v);
+                amax = fmaxf(amax, fabsf(r));
+                c1[k] += v;
+                c2[k] += r - v;
+            }
+#pragma unroll
+            for (int off = 1; off < 4; off <<= 1) {
+                c1[k] += __shfl_xor_sync(0xffffffffu, c1[k], off);
+                c2[k] += __shfl_xor_sync(0xffffffffu, c2[k], off);
+            }
+        }
+#pragma unroll
+        for (int off = 1; off < 4; off <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
+        // scaled by the power of two that takes the largest value into [2^14, 2^15)
+        int E = (int)(__float_as_uint(amax) >> 23);
+        E = E < 20 ? 20 : (E > 230 ? 230 : E);
+        const float up = __uint_as_float((uint32_t)(268 - E) << 23);
+        if (warp == 0 && t == 0 && (Q8 || g < 4)) {
+            float* st = stat + qi * (2 * NB + 1);
+#pragma unroll
+            for (int k = 0; k < NB; k++) {  // in the unit of D, 2^24 / up
+                st[2 * k] = c1[k] * up * 5.9604645e-08f;
+                st[2 * k + 1] = kOff * c2[k] * up * 5.9604645e-08f;
+            }
+            st[2 * NB] = __uint_as_float((uint32_t)(E + 10) << 23) * kLog2e;
+        }
+        for (int s = 2 * warp; s < 2 * warp + 2; s++) {  // two of the eight MMA steps per warp
+            const int k = s / kKs, ks = s % kKs;
+            uint32_t wh[2], wl[2];
+#pragma unroll
+            for (int hf = 0; hf < 2; hf++) {
+                const int p = 2 * ks + hf, i = p % kCL, c0 = (p / kCL) * 2 * kCL + i;
+                const float down = up * __uint_as_float((uint32_t)(127 - code_shift<BITS>(i)) << 23);
+                const int ch = k * kBlk + t * kKC + c0;
+                split_f16(rounded(value(ch)) * down, rounded(value(ch + kCL)) * down, wh[hf], wl[hf]);
+            }
+            if (Q8) {
+                qb[32 * s] = make_uint4(wh[0], wh[1], wl[0], wl[1]);
+            } else {
+                const bool high = g < 4;
+                qb[32 * s] = make_uint4(high ? wh[0] : wl[0], high ? wh[1] : wl[1], 0u, 0u);
+            }
+        }
+    }
+    __syncthreads();
+
+    // this lane's score columns 2t, 2t + 1: queries q0, q0 + 1 (columns 4..7 without Q8: their low
+    // parts, which take no C terms)
+    const int q0 = Q8 ? 2 * t : 2 * (t & 1);
+    const bool main_cols = Q8 || t < 2;
+    float2 cblk[NB], eblk[NB], cF;
+#pragma unroll
+    for (int k = 0; k < NB; k++) {
+        const float* s0 = stat + q0 * (2 * NB + 1) + 2 * k;
+        cblk[k] = main_cols ? make_float2(s0[0], s0[2 * NB + 1]) : dup(0.0f);
+        eblk[k] = main_cols ? make_float2(s0[1], s0[2 * NB + 2]) : dup(0.0f);
+    }
+    cF = make_float2(stat[q0 * (2 * NB + 1) + 2 * NB], stat[(q0 + 1) * (2 * NB + 1) + 2 * NB]);
+
+    // columns 2t, 2t + 1: sums of w q over channels (code i of lane g's segment in pass p)
+    float2 acc[kPass][kVC];
+#pragma unroll
+    for (int p = 0; p < kPass; p++)
+#pragma unroll
+        for (int i = 0; i < kVC; i++) acc[p][i] = dup(0.0f);
+    float2 Mu = dup(-INFINITY), lsum = dup(0.0f), zsum[NB];
+#pragma unroll
+    for (int k = 0; k < NB; k++) zsum[k] = dup(0.0f);
+    int kb = 0;  // the weights carry a factor 2^kb (their low parts stay in fp16's normal range)
+
+    for (int it = 0; it < steps; it++) {
+        const uint32_t par = (phase + (uint32_t)it) & 1u;
+        const int n_tok = step_tokens(it);
+        // this step's scales to shared memory as fp32, the next step's on their way
+#pragma unroll
+        for (int s = 0; s < 2; s++)
+#pragma unroll
+            for (int e = 0; e < kItems; e++) {
+                const float2 z = scale_zero_of(nsc[s][e]);
+                sf[s * C::kRecs + lane + 32 * e] = make_float4(z.x, z.x, z.y, z.y);
+            }
+        if (it + 1 < steps) load_scales(it + 1);
+        bool ok = mbar_wait(&bars[0], par, abort_flag, a.wait_ns);
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) raise_flag(a.status, CG_FLAG_PIPE_TIMEOUT);
+            mbar_wait(&bars[0], par, abort_flag + 1, tc::kWaitLimitNs);  // let the copies in flight land
+            mbar_wait(&bars[1], par, abort_flag + 1, tc::kWaitLimitNs);
+            dead = true;
+            break;
+        }
+        __syncwarp();
+        const float4* SK = sf + tg * NB;
+        const float4* SV = sf + C::kRecs + tg * NB;
+
+        // ---- scores: S[j][h] = tokens 16 j + 8 h + tg, two queries
+        float2 S[kTiles][2];
+#pragma unroll
+        for (int j = 0; j < kTiles; j++) S[j][0] = S[j][1] = dup(0.0f);
+#pragma unroll
+        for (int k = 0; k < NB; k++) {
+            uint32_t x[kTiles][2][kKX];
+            float d[kTiles][4];
+#pragma unroll
+            for (int j = 0; j < kTiles; j++) {
+#pragma unroll
+                for (int hf = 0; hf < 2; hf++) {
+                    const unsigned char* src = kst + (16 * j + 8 * hf + tg) * C::kRow + (k * kBlk + t * kKC) * BITS / 8;
+                    uint32_t(&w)[kKX] = x[j][hf];
+                    if constexpr (kLaneBits == 8) {
+                        w[0] = __byte_perm(*reinterpret_cast<const uint16_t*>(src), 0u, 0x4140);
+                    } else if constexpr (kKX % 4 == 0) {
+#pragma unroll
+                        for (int q = 0; q < kKX; q += 4) {
+                            const uint4 v = reinterpret_cast<const uint4*>(src)[q / 4];
+                            w[q] = v.x; w[q + 1] = v.y; w[q + 2] = v.z; w[q + 3] = v.w;
+                        }
+                    } else if constexpr (kKX == 2) {
+                        const uint2 v = *reinterpret_cast<const uint2*>(src);
+                        w[0] = v.x; w[1] = v.y;
+                    } else {
+                        w[0] = *reinterpret_cast<const uint32_t*>(src);
+                    }
+                }
+                d[j][0] = d[j][1] = d[j][2] = d[j][3] = 0.0f;
+            }
+#pragma unroll
+            for (int ks = 0; ks < kKs; ks++) {
+                uint4 q;
+                if constexpr (Q8) {
+                    q = qb[32 * (k * kKs + ks)];
+                } else {
+                    const uint2 v = *reinterpret_cast<const uint2*>(&qb[32 * (k * kKs + ks)]);
+                    q = make_uint4(v.x, v.y, 0u, 0u);
+                }
+                const int p0 = 2 * ks, p1 = 2 * ks + 1;
+#pragma unroll
+                for (int j = 0; j < kTiles; j++) {
+                    const uint32_t a0 = code_pair<BITS>(x[j][0][p0 / kCL], p0 % kCL);
+                    const uint32_t a1 = code_pair<BITS>(x[j][1][p0 / kCL], p0 % kCL);
+                    const uint32_t a2 = code_pair<BITS>(x[j][0][p1 / kCL], p1 % kCL);
+                    const uint32_t a3 = code_pair<BITS>(x[j][1][p1 / kCL], p1 % kCL);
+                    mma_f16(d[j], a0, a1, a2, a3, q.x, q.y);
+                    if constexpr (Q8) mma_f16(d[j], a0, a1, a2, a3, q.z, q.w);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kTiles; j++)
+#pragma unroll
+                for (int hf = 0; hf < 2; hf++) {
+                    const float4 z = SK[(16 * j + 8 * hf) * NB + k];
+                    float2 u = make_float2(d[j][2 * hf], d[j][2 * hf + 1]);
+                    if constexpr (BITS != 8) u = __fadd2_rn(u, eblk[k]);
+                    S[j][hf] = __ffma2_rn(make_float2(z.z, z.w), cblk[k], S[j][hf]);
+                    S[j][hf] = __ffma2_rn(make_float2(z.x, z.y), u, S[j][hf]);
+                }
+        }
+        __syncwarp();  // all lanes have read the key codes
+        if (lane == 0 && it + 1 < steps) load_codes(it + 1, 0);
+        if constexpr (!Q8) {  // high + low columns
+#pragma unroll
+            for (int j = 0; j < kTiles; j++)
+#pragma unroll
+                for (int hf = 0; hf < 2; hf++)
+                    S[j][hf] = __fadd2_rn(S[j][hf], make_float2(__shfl_xor_sync(0xffffffffu, S[j][hf].x, 2),
+                                                                __shfl_xor_sync(0xffffffffu, S[j][hf].y, 2)));
+        }
+        if (n_tok < kTok) {
+#pragma unroll
+            for (int j = 0; j < kTiles; j++)
+#pragma unroll
+                for (int hf = 0; hf < 2; hf++)
+                    if (16 * j + 8 * hf + tg >= n_tok) S[j][hf] = dup(-INFINITY);
+        }
+
+        // ---- online softmax of this warp's stream (the lanes of a column agree)
+        float2 m = S[0][0];
+#pragma unroll
+        for (int j = 0; j < kTiles; j++)
+#pragma unroll
+            for (int hf = 0; hf < 2; hf++) {
+                m.x = fmaxf(m.x, S[j][hf].x);
+                m.y = fmaxf(m.y, S[j][hf].y);
+            }
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+            m.x = fmaxf(m.x, __shfl_xor_sync(0xffffffffu, m.x, off));
+            m.y = fmaxf(m.y, __shfl_xor_sync(0xffffffffu, m.y, off));
+        }
+        if (it == 0) {
+            float smax = 0.0f;
+            for (int e = 0; e < kTok / 8 * NB; e++) smax = fmaxf(smax, SV[(e / NB) * 8 * NB + e % NB].x);
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, off));
+            const int e = (int)(__float_as_uint(smax) >> 23) - 127;
+            kb = smax > 0.0f && e < 8 ? 8 - e : 0;
+        }
+        m.x = fmaxf(Mu.x, m.x);
+        m.y = fmaxf(Mu.y, m.y);
+        const float2 al = make_float2(ex2((Mu.x - m.x) * cF.x), ex2((Mu.y - m.y) * cF.y));  // 0 on the first step
+        Mu = m;
+        const float2 bias = make_float2((float)kb - m.x * cF.x, (float)kb - m.y * cF.y);
+        float2 l2 = dup(0.0f);
+#pragma unroll
+        for (int j = 0; j < kTiles; j++)
+#pragma unroll
+            for (int hf = 0; hf < 2; hf++) {
+                const float2 e = __ffma2_rn(S[j][hf], cF, bias);
+                S[j][hf] = make_float2(ex2(e.x), ex2(e.y));
+                l2 = __fadd2_rn(l2, S[j][hf]);
+            }
+        lsum = __ffma2_rn(lsum, al, l2);
+
+        ok = mbar_wait(&bars[1], par, abort_flag, a.wait_ns);
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) raise_flag(a.status, CG_FLAG_PIPE_TIMEOUT);
+            mbar_wait(&bars[1], par, abort_flag + 1, tc::kWaitLimitNs);
+            if (it + 1 < steps) mbar_wait(&bars[0], par ^ 1u, abort_flag + 1, tc::kWaitLimitNs);
+            dead = true;
+            break;
+        }
+
+        // ---- values: pass by pass (a pass lies in one block), 16 tokens per MMA
+        uint32_t wb[kTiles][Q8 ? 4 : 2];  // weights: rows 0..7, 8..15 of the sixteen tokens (Q8: high, then low)
+#pragma unroll
+        for (int p = 0; p < kPass; p++) {
+            const int k = NB == 1 ? 0 : p;
+            if (NB > 1 || p == 0) {
+                for (;;) {
+                    float2 z2 = dup(0.0f);
+                    __half2 top = __float2half2_rn(0.0f);
+#pragma unroll
+                    for (int j = 0; j < kTiles; j++)
+#pragma unroll
+                        for (int hf = 0; hf < 2; hf++) {
+                            const float4 z = SV[(16 * j + 8 * hf) * NB + k];
+                            z2 = __ffma2_rn(S[j][hf], make_float2(z.z, z.w), z2);
+                            const float2 w2 = __fmul2_rn(S[j][hf], make_float2(z.x, z.y));
+                            uint32_t wh, wl;
+                            split_f16(w2.x, w2.y, wh, wl);
+                            top = __hmax2(top, *reinterpret_cast<const __half2*>(&wh));
+                            if constexpr (Q8) {
+                                wb[j][hf] = transpose8x8(wh);
+                                wb[j][2 + hf] = transpose8x8(wl);
+                            } else {
+                                wb[j][hf] = transpose8x8(main_cols ? wh : wl);
+                            }
+                        }
+                    // weights above fp16 (a value scale far above the first step's): drop the factor 2^kb
+                    const bool over = __hisinf(__low2half(top)) || __hisinf(__high2half(top));
+                    if (kb == 0 || !__any_sync(0xffffffffu, over)) {
+                        zsum[k] = __ffma2_rn(zsum[k], al, z2);
+                        break;
+                    }
+                    const float2 f = dup(__uint_as_float((uint32_t)(127 - kb) << 23));
+                    kb = 0;
+                    lsum = __fmul2_rn(lsum, f);
+#pragma unroll
+                    for (int q = 0; q < NB; q++) zsum[q] = __fmul2_rn(zsum[q], f);
+#pragma unroll
+                    for (int q = 0; q < kPass; q++)
+#pragma unroll
+                        for (int i = 0; i < kVC; i++) acc[q][i] = __fmul2_rn(acc[q][i], f);
+#pragma unroll
+                    for (int j = 0; j < kTiles; j++) {
+                        S[j][0] = __fmul2_rn(S[j][0], f);
+                        S[j][1] = __fmul2_rn(S[j][1], f);
+                    }
+                }
+            }
+            float d[kVC / 2][4];  // channels of codes 2 m and 2 m + 1
+#pragma unroll
+            for (int m2 = 0; m2 < kVC / 2; m2++) d[m2][0] = d[m2][1] = d[m2][2] = d[m2][3] = 0.0f;
+            const unsigned char* vbase = vst + (NB == 1 ? 2 * g + p : 8 * p + g) * kVBits / 8;
+#pragma unroll
+            for (int j = 0; j < kTiles; j++) {
+                // tokens t, t + 4, t + 8, t + 12 of the sixteen: MMA columns 2t, 2t + 1, 2t + 8, 2t + 9
+                uint32_t w[4][kVX > 2 ? 2 : 1];
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const unsigned char* src = vbase + (16 * j + t + 4 * q) * C::kRow;
+                    if constexpr (kVBits == 64) {
+                        const uint2 v = *reinterpret_cast<const uint2*>(src);
+                        w[q][0] = v.x;
+                        w[q][kVX > 2 ? 1 : 0] = v.y;
+                    } else if constexpr (kVBits == 32) {
+                        w[q][0] = *reinterpret_cast<const uint32_t*>(src);
+                    } else if constexpr (kVBits == 16) {
+                        w[q][0] = *reinterpret_cast<const uint16_t*>(src);
+                    } else {
+                        w[q][0] = *src;
+                    }
+                }
+#pragma unroll
+                for (int x = 0; x < kVX; x++) {
+                    const uint32_t sel = x & 1 ? 0x7632u : 0x5410u;
+                    const uint32_t y0 = __byte_perm(w[0][x >> 1], w[1][x >> 1], sel);
+                    const uint32_t y1 = __byte_perm(w[2][x >> 1], w[3][x >> 1], sel);
+#pragma unroll
+                    for (int i = 0; i < kVL; i += 2) {
+                        float(&dd)[4] = d[(x * kVL + i) / 2];
+                        const uint32_t a0 = code_pair<BITS>(y0, i), a1 = code_pair<BITS>(y0, i + 1);
+                        const uint32_t a2 = code_pair<BITS>(y1, i), a3 = code_pair<BITS>(y1, i + 1);
+                        mma_f16(dd, a0, a1, a2, a3, wb[j][0], wb[j][1]);
+                        if constexpr (Q8) mma_f16(dd, a0, a1, a2, a3, wb[j][2], wb[j][3]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kVC; i++)
+                acc[p][i] = __ffma2_rn(acc[p][i], al, make_float2(d[i / 2][2 * (i & 1)], d[i / 2][2 * (i & 1) + 1]));
+        }
+        __syncwarp();  // all lanes have read the value codes and the scales
+        if (lane == 0 && it + 1 < steps) load_codes(it + 1, 1);
+    }
+    phase += (uint32_t)steps;
+
+    // ---- the part: four warp streams merged in shared memory (the buffers are free)
+#pragma unroll
+    for (int off = 4; off < 32; off <<= 1) {
+        lsum.x += __shfl_xor_sync(0xffffffffu, lsum.x, off);
+        lsum.y += __shfl_xor_sync(0xffffffffu, lsum.y, off);
+#pragma unroll
+        for (int k = 0; k < NB; k++) {
+            zsum[k].x += __shfl_xor_sync(0xffffffffu, zsum[k].x, off);
+            zsum[k].y += __shfl_xor_sync(0xffffffffu, zsum[k].y, off);
+        }
+    }
+    __syncthreads();
+    float* mo = reinterpret_cast<float*>(smem + C::kFixed);  // [warp][query][128]
+    float* ml = mo + kSWarps * 8 * kAD;                      // [warp][query][max (log2), sum]
+    const float unscale = __uint_as_float((uint32_t)(127 - kb) << 23);
+#pragma unroll
+    for (int p = 0; p < kPass; p++)
+#pragma unroll
+        for (int i = 0; i < kVC; i++) {
+            const float f = 16777216.0f / (float)(1 << code_shift<BITS>(i % kVL));
+            const int ch = NB == 1 ? 16 * g + kVC * p + i : kBlk * p + kVC * g + i;
+            float2 v = acc[p][i];
+            if constexpr (!Q8) {
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, 2);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, 2);
+            }
+            if (main_cols) {
+                const float2 z = zsum[NB == 1 ? 0 : p];
+                mo[(warp * 8 + q0) * kAD + ch] = fmaf(v.x, f, z.x) * unscale;
+                mo[(warp * 8 + q0 + 1) * kAD + ch] = fmaf(v.y, f, z.y) * unscale;
+            }
+        }
+    if (g == 0 && main_cols) {
+        float* s0 = ml + (warp * 8 + q0) * 2;
+        s0[0] = steps > 0 ? Mu.x * cF.x : -INFINITY;
+        s0[1] = lsum.x * unscale;
+        s0[2] = steps > 0 ? Mu.y * cF.y : -INFINITY;
+        s0[3] = lsum.y * unscale;
+    }
+    __syncthreads();
+    float* part = a.part + ((int64_t)unit * a.n_parts + slot) * a.n_rep * (kAD + 2);
+    for (int r = 0; r < a.n_rep; r++) {
+        float M = ml[r * 2];  // warp 0 has at least one step
+        for (int w = 1; w < kSWarps; w++) M = fmaxf(M, ml[(w * 8 + r) * 2]);
+        float o = 0.0f, ls = 0.0f;
+        for (int w = 0; w < kSWarps; w++) {
+            const float mw = ml[(w * 8 + r) * 2];
+            if (mw == -INFINITY) continue;  // a stream without tokens
+            const float e = ex2(mw - M);
+            ls = fmaf(ml[(w * 8 + r) * 2 + 1], e, ls);
+            o = fmaf(mo[(w * 8 + r) * kAD + tid], e, o);
+        }
+        part[r * (kAD + 2) + 2 + tid] = o;
+        if (tid == 0) {
+            part[r * (kAD + 2)] = M;
+            part[r * (kAD + 2) + 1] = ls;
+        }
+    }
+    // the buffers go back to the copies of the next segment
+    fence_proxy_async_smem();
+    __syncthreads();
+    }
+}
+
+// Launches a kernel that may start while the one before it in the stream still runs; it waits
+// (griddepcontrol.wait) before it reads what that one wrote.
+template <typename K>
+cudaError_t launch_dependent(K kernel, unsigned grid, unsigned threads, size_t smem, const AttnArgs& a, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+template <int BITS, int NB, bool Q8>
+cudaError_t launch_stream(AttnArgs& a, int sms, cudaStream_t st) {
+    using C = StreamCfg<BITS, NB>;
+    cudaError_t e = cudaFuncSetAttribute(attn_stream_kernel<BITS, NB, Q8>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kTotal);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)a.n_parts, (unsigned)(a.L * a.B * a.H));
-    attn_chunk_mma_kernel<BITS, NREP><<<grid, kMThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    // All units' steps in equal shares over the CTAs that fit at once: a share starts and ends
+    // anywhere in a unit, so no SM waits for a last wave (64 sequences x 8 heads: 72 steps a CTA; whole
+    // parts per CTA took 5 waves of 18). A unit's parts lie on consecutive CTAs.
+    const int64_t units = (int64_t)a.L * a.B * a.H, slots = (int64_t)sms * kSCtas;
+    a.unit_steps = (a.T + kSWarps * C::kTok - 1) / (kSWarps * C::kTok);
+    a.all_steps = units * a.unit_steps;
+    a.cta_steps = (a.all_steps + slots - 1) / slots;
+    const int64_t most = (a.unit_steps + a.cta_steps - 1) / a.cta_steps + 1;
+    a.n_parts = (int)(most < a.unit_steps ? most : a.unit_steps);  // at most one per 128 tokens (the workspace)
+    const int64_t grid = (a.all_steps + a.cta_steps - 1) / a.cta_steps;
+    return launch_dependent(attn_stream_kernel<BITS, NB, Q8>, (unsigned)grid, kSThreads, C::kTotal, a, st);
 }
 
 template <int BITS>
-cudaError_t launch_mma_bits(const AttnArgs& a, cudaStream_t st) {
-    switch (a.n_rep) {
-        case 1: return launch_mma_chunks<BITS, 1>(a, st);
-        case 2: return launch_mma_chunks<BITS, 2>(a, st);
-        case 4: return launch_mma_chunks<BITS, 4>(a, st);
-        case 8: return launch_mma_chunks<BITS, 8>(a, st);
-        default: return cudaErrorInvalidValue;
-    }
+cudaError_t launch_stream_bits(AttnArgs& a, int sms, cudaStream_t st) {
+    const bool q8 = a.n_rep > 4;
+    if (a.blk == 128) return q8 ? launch_stream<BITS, 1, true>(a, sms, st) : launch_stream<BITS, 1, false>(a, sms, st);
+    if (a.blk == 64) return q8 ? launch_stream<BITS, 2, true>(a, sms, st) : launch_stream<BITS, 2, false>(a, sms, st);
+    return q8 ? launch_stream<BITS, 4, true>(a, sms, st) : launch_stream<BITS, 4, false>(a, sms, st);
 }
 
 template <int BITS, int NREP>
@@ -781,37 +1050,34 @@ size_t attn_workspace_bytes(int64_t units, int n_rep, int d, int64_t T) {
 
 cudaError_t launch_attention(const AttnArgs& args, cudaStream_t st) {
     AttnArgs a = args;
-    const bool mma = a.bits == 2 || a.bits == 4;
-    if (mma) {
-        // parts of consecutive chunks per (l, b, h): enough CTAs to fill the SMs a few times over
-        int dev = 0, sms = 152;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int64_t units = (int64_t)a.L * a.B * a.H, target = (int64_t)sms * 12;
-        int64_t splits = (target + units - 1) / units;
-        if (splits > a.n_chunks) splits = a.n_chunks;
-        if (splits < 1) splits = 1;
-        a.chunks_per_part = (int)((a.n_chunks + splits - 1) / splits);
-        a.n_parts = (a.n_chunks + a.chunks_per_part - 1) / a.chunks_per_part;
-    } else {
-        a.chunks_per_part = 1;
-        a.n_parts = a.n_chunks;
-    }
-    const size_t gsmem = (size_t)kAD * a.g * 4 + kAD * 4;
-    cudaError_t e = cudaFuncSetAttribute(attn_query_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem);
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int queries = a.B * a.n_rep;
+    const size_t qsmem = (size_t)(kAD * (a.g + 4) + kQueries * kAD) * 4;
+    cudaError_t e = cudaFuncSetAttribute(attn_query_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qsmem);
     if (e != cudaSuccess) return e;
-    attn_query_kernel<<<dim3((unsigned)(a.L * a.H), (unsigned)((a.B + kQuerySeqs - 1) / kQuerySeqs)), kAD, gsmem, st>>>(a);
+    attn_query_kernel<<<dim3((unsigned)(a.L * a.H), (unsigned)((queries + kQueries - 1) / kQueries)), kQThreads, qsmem, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    a.n_parts = a.n_chunks;  // 3 and 6 bits: one chunk per part
+    a.unit_steps = a.n_chunks;
+    a.cta_steps = 1;
     switch (a.bits) {
-        case 2: e = launch_mma_bits<2>(a, st); break;
+        case 2: e = launch_stream_bits<2>(a, sms, st); break;
         case 3: e = launch_chunks_bits<3>(a, st); break;
-        case 4: e = launch_mma_bits<4>(a, st); break;
+        case 4: e = launch_stream_bits<4>(a, sms, st); break;
         case 6: e = launch_chunks_bits<6>(a, st); break;
-        case 8: e = launch_chunks_bits<8>(a, st); break;
+        case 8: e = launch_stream_bits<8>(a, sms, st); break;
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    attn_combine_kernel<<<(unsigned)(a.L * a.B * a.H), kAD, 0, st>>>(a);
-    return cudaGetLastError();
+    const unsigned units = (unsigned)(a.L * a.B * a.H);
+    switch (a.n_rep) {
+        case 1: return launch_dependent(attn_combine_kernel<1>, units, kCThreads, 0, a, st);
+        case 2: return launch_dependent(attn_combine_kernel<2>, units, kCThreads, 0, a, st);
+        case 4: return launch_dependent(attn_combine_kernel<4>, units, kCThreads, 0, a, st);
+        case 8: return launch_dependent(attn_combine_kernel<8>, units, kCThreads, 0, a, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace cg

@@ -77,9 +77,11 @@ struct AttnArgs {
     float* out;             // fp32 [L][B][H][n_rep][d]
     int L, B, H, d, g, bits, blk, n_rep;
     int64_t T;              // tokens attended
-    int n_chunks;           // 256-token chunks of [t0, t0 + T)
-    int n_parts;            // partial results per (l, b, h), each over chunks_per_part chunks
-    int chunks_per_part;
+    int n_chunks;           // 128-token chunks of [t0, t0 + T)
+    int n_parts;            // room for partial results per (l, b, h), at most n_chunks
+    // Steps (token groups) of one (l, b, h), of all and of one CTA: CTA c takes steps
+    // [c, c + 1) * cta_steps of the units' steps in order, one partial result per unit it meets
+    int64_t unit_steps, all_steps, cta_steps;
     float scale;
     int32_t* status;
     uint64_t wait_ns;       // limit of the bounded waits on the chunk copies
