@@ -116,6 +116,17 @@ __host__ __device__ constexpr uint32_t pack_bias(int w) {
     return k;
 }
 
+// BITS-bit code of z~ in the packed word set of a 32-code chunk: y = 0x4B400000 + q is added
+// shifted to its bit offset (wrapping sums; the constant part is removed at the end), the
+// high bits of a code that straddles two words go to the next word.
+template <int BITS>
+__device__ __forceinline__ void put_code(uint32_t (&words)[BITS], int k, uint32_t y) {
+    constexpr uint32_t qmask = (1u << BITS) - 1u;
+    const int bit = k * BITS;
+    words[bit >> 5] += y << (bit & 31);
+    if ((bit & 31) + BITS > 32) words[(bit >> 5) + 1] += (y & qmask) >> (32 - (bit & 31));
+}
+
 __device__ __forceinline__ uint32_t scale16(float mx, float mn, float qmax) {
     return f2h_bits(__fdiv_rn(__fsub_rn(mx, mn), qmax));
 }

@@ -185,17 +185,6 @@ __device__ __forceinline__ float half_warp_max(float v) {
     return v;
 }
 
-// BITS-bit code of z~ in the packed word set of a 32-code chunk: y = 0x4B400000 + q is added
-// shifted to its bit offset (wrapping sums; the constant part is removed at the end), the
-// high bits of a code that straddles two words go to the next word.
-template <int BITS>
-__device__ __forceinline__ void put_code(uint32_t (&words)[BITS], int k, uint32_t y) {
-    constexpr uint32_t qmask = (1u << BITS) - 1u;
-    const int bit = k * BITS;
-    words[bit >> 5] += y << (bit & 31);
-    if ((bit & 31) + BITS > 32) words[(bit >> 5) + 1] += (y & qmask) >> (32 - (bit & 31));
-}
-
 template <int BITS, int NBK, bool TILE>
 __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __grid_constant__ CUtensorMap xmap,
                                                                       const RowEncParams P) {

@@ -41,4 +41,19 @@ inline bool make_tmap_bf16_sw128(CUtensorMap* map, const void* base, uint64_t ro
     return r == CUDA_SUCCESS;
 }
 
+// bf16 tensor as [rows][32] (64-byte rows), moved in boxes of 32 rows with the 64-byte swizzle;
+// out-of-range rows read as 0 and are not written.
+inline bool make_tmap_bf16_rows32(CUtensorMap* map, const void* base, uint64_t rows) {
+    auto fn = tmap_encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[2] = {32, rows};
+    cuuint64_t strides[1] = {64};
+    cuuint32_t box[2] = {32, 32};
+    cuuint32_t estr[2] = {1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 }  // namespace cg
