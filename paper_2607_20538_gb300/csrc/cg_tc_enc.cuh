@@ -59,7 +59,7 @@ __host__ __device__ __forceinline__ void bound_range(int bk, int g, int blk, int
 }
 
 // One warp-wide round of exact recomputation of the queued gauge-space values (job word:
-// row | col << 8; the value goes to the next word), in the library's fixed order. A team
+// row | col << 8 | flags << 16; value c goes to res[c]), in the library's fixed order. A team
 // of T = g/4 lanes computes one value: lane j forms the products of channels 4j..4j+3 and
 // their pairwise sum, and the team combines its partial sums with xor-shuffles, which
 // follows the same pairwise tree. Each lane loads the operands of kSlots values before any
@@ -67,8 +67,8 @@ __host__ __device__ __forceinline__ void bound_range(int bk, int g, int blk, int
 // staged bf16 tile (two 64-column halves, 128-byte swizzle), Gf the gauge set in global
 // memory.
 template <int kSlots>
-__device__ __forceinline__ void run_jobs(uint32_t* qjob, int nq, const unsigned char* stage, const float* Gf, int g,
-                                      int lane) {
+__device__ __forceinline__ void run_jobs(const uint32_t* jobs, float* res, int nq, const unsigned char* stage,
+                                         const float* Gf, int g, int lane) {
     const int lgT = 29 - __clz(g);  // log2(g / 4); g in {8, ..., 128}
     const int T = 1 << lgT, teams = 32 >> lgT;
     const int tm = lane >> lgT, j = lane & (T - 1);
@@ -78,7 +78,7 @@ __device__ __forceinline__ void run_jobs(uint32_t* qjob, int nq, const unsigned 
 #pragma unroll
         for (int k = 0; k < kSlots; k++) {
             const int c = base + k * teams + tm;
-            const uint32_t jb = qjob[2 * (c < nq ? c : 0)];
+            const uint32_t jb = jobs[c < nq ? c : 0];
             const int row = (int)(jb & 0xffu), col = (int)((jb >> 8) & 0xffu);
             const int kk = (col & ~(g - 1)) + 4 * j;  // first channel of this lane's products
             xv[k] = *reinterpret_cast<const uint2*>(stage + (kk >> 6) * 16384 + row * 128 +
@@ -100,7 +100,7 @@ __device__ __forceinline__ void run_jobs(uint32_t* qjob, int nq, const unsigned 
 #pragma unroll
             for (int k = 0; k < kSlots; k++) {
                 const int c = base + k * teams + tm;
-                if (c < nq) qjob[2 * c + 1] = __float_as_uint(part[k]);
+                if (c < nq) res[c] = part[k];
             }
         }
     }

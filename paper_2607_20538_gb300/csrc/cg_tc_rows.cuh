@@ -28,7 +28,10 @@
 //      (both are monotone in the extremes, so equal interval ends decide them exactly);
 //   4. blocks the intervals leave undecided: candidate extremes (values within 2E of the
 //      approximate extreme, only in chunks whose own extreme qualifies) are recomputed
-//      exactly in the library's order by the warp together (run_jobs);
+//      exactly in the library's order by the warp together (run_jobs). A warp has one or two
+//      such rows a tile; a row's chunk is spread over the lanes through 128 bytes of shared
+//      memory, so one compare and vote finds its candidates (building a 32-bit candidate mask
+//      in every lane, and job lists by prefix sums over them, took twice the instructions);
 //   5. codes straight from tensor memory: t = z~ * (1/s) - m/s, y = t + 1.5 * 2^23 (round to
 //      nearest even in the add; y's bit pattern is 0x4B400000 + q), packed by wrapping sums
 //      of y << (bit offset) less a compile-time constant. A chunk takes the short loop when
@@ -66,14 +69,15 @@ constexpr int kThreads = 640;
 constexpr int kEpiWG = 4;  // epilogue warpgroups
 constexpr int kConvWarp1 = 19;  // second gauge-converter warp (the first is warp 2)
 constexpr int kEpiWarp0 = 3;
-constexpr int kQCap = 20;  // repair jobs per warp and round
+constexpr int kJobCap = 8;  // exact recomputes per warp and round
 constexpr int kAcc = 4;    // accumulator buffers in tensor memory
 
 struct RowSmem {
     static constexpr uint32_t stages = 0;
     static constexpr uint32_t bsplit = stages + kStages * kTileBytes;  // 3 x (16 or 32 KB)
-    static constexpr uint32_t queue = bsplit + kNPass * 32768;         // 16 warps x kQCap x 8 B
-    static constexpr uint32_t misc = queue + 4 * kEpiWG * kQCap * 8;
+    static constexpr uint32_t warp_buf = 128 + kJobCap * 4;            // a 32-value row chunk or results; jobs
+    static constexpr uint32_t bufs = bsplit + kNPass * 32768;          // 16 epilogue warps
+    static constexpr uint32_t misc = bufs + 4 * kEpiWG * warp_buf;
     static constexpr uint32_t total = misc + 512;  // base is 1024-aligned (checked in-kernel)
 };
 
@@ -198,7 +202,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
     RowMisc* M = reinterpret_cast<RowMisc*>(sm + RowSmem::misc);
     unsigned char* stages = sm + RowSmem::stages;
     unsigned char* bsplit = sm + RowSmem::bsplit;
-    uint32_t* queue = reinterpret_cast<uint32_t*>(sm + RowSmem::queue);
 
     const RowArgs& a = P.a;
     const tc::Sched& S = P.S;
@@ -366,13 +369,37 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
         const int wg = (warp - kEpiWarp0) >> 2;  // warpgroup: tiles i = wg (mod kEpiWG)
         const int q4 = warp & 3;                 // TMEM lane quadrant of this warp
         const int row = q4 * 32 + lane;          // TMEM lane = token row of the tile
-        const int qw = warp - kEpiWarp0;         // job queue of this warp
-        uint32_t* qjob = queue + qw * kQCap * 2;
+        float* rowbuf = reinterpret_cast<float*>(sm + RowSmem::bufs + (warp - kEpiWarp0) * RowSmem::warp_buf);
+        uint32_t* jobs = reinterpret_cast<uint32_t*>(rowbuf + 32);
+        const uint32_t lt = (1u << lane) - 1u;
+        // Row chunk of lane `src` (its 32 values v) spread over the lanes: lane k gets value k.
+        auto spread = [&](const uint32_t (&v)[32], int src) -> float {
+            __syncwarp();
+            if (lane == src) {
+#pragma unroll
+                for (int k = 0; k < 32; k += 4)
+                    *reinterpret_cast<uint4*>(rowbuf + k) = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+            }
+            __syncwarp();
+            return rowbuf[lane];
+        };
+        // Appends a job for every set lane of m (column 32 c + lane of row src) while there is room;
+        // returns the lanes left over.
+        auto append = [&](uint32_t m, uint32_t word, int& nj) -> uint32_t {
+            const bool mine = (m >> lane) & 1u;
+            const int at = nj + __popc(m & lt);
+            if (mine && at < kJobCap) jobs[at] = word;
+            const int n = nj + __popc(m);
+            nj = n < kJobCap ? n : kJobCap;
+            return n > kJobCap ? __ballot_sync(0xffffffffu, mine && at >= kJobCap) : 0u;
+        };
         constexpr float qmaxf = (float)((1 << BITS) - 1);
         constexpr float kRq = 1.0f / qmaxf;        // fl(1 / qmax)
         constexpr float kBelow1 = 1.0f - 8.0f * kU;  // 1 - 2^-21 and 1 + 2^-21, both exact in fp32
         constexpr float kAbove1 = 1.0f + 8.0f * kU;
         constexpr int qmax = (1 << BITS) - 1;
+        // 8-bit codes nearly always have mu >= 1e-4: their usual loop tracks the distances too
+        constexpr bool kTrack = TILE || BITS == 8;
         constexpr int kJobSlots = NBK == 2 ? 4 : 2;  // values per lane and memory round trip
         int32_t flag = 0;
         tc::TileIter it;
@@ -490,114 +517,67 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                 if (valid && mlo != mhi) amb |= 2 << (2 * bk);
             }
 
-            // ---- 4. exact extremes of undecided blocks (warp-cooperative rounds)
+            // ---- 4. exact extremes of undecided blocks. Candidates of a block's min (max) are its values
+            // within 2E of the approximate min (max), only in chunks whose own min (max) lies that close.
+            // The few rows concerned are taken one by one: the row's chunk is spread over the lanes, so
+            // that one compare and vote finds its candidates
             if (__any_sync(0xffffffffu, amb != 0)) {
-                // candidates of an undecided block's min (max): its values within 2E of the
-                // approximate min (max), only in chunks whose own min (max) lies that close
-                uint32_t pm[4] = {0, 0, 0, 0}, px[4] = {0, 0, 0, 0};
-#pragma unroll 1
-                for (int c = 0; c < 4; c++) {
-                    const int bk = c / CPB;
-                    const int need = (amb >> (2 * bk)) & 3;
-                    const float e2 = 2.0f * pickn(E, bk);
-                    const float tl = __fadd_rn(pickn(mn, bk), e2), th = __fsub_rn(pickn(mx, bk), e2);
-                    const bool nl = need != 0 && pickn(cmn, c) <= tl;
-                    const bool nh = (need & 1) && pickn(cmx, c) >= th;
-                    uint32_t m0 = 0, m1 = 0;
-                    const bool anyl = __any_sync(0xffffffffu, nl), anyh = __any_sync(0xffffffffu, nh);
-                    if (anyl || anyh) {
-                        uint32_t v[32];
-                        tmem_ld32(tacc + c * 32, v);
-                        tmem_wait_ld();
-                        // sign bits of tl - z (z > tl) and z - th (z < th), one bit per column;
-                        // each side only when some lane of the warp needs it (with four blocks
-                        // per row, one loop for both keeps the row's state in registers)
-                        uint32_t a0 = 0, a1 = 0;
-                        if constexpr (NBK == 4) {
-#pragma unroll
-                            for (int k = 31; k >= 0; k--) {
-                                const float z = __uint_as_float(v[k]);
-                                a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl, z)), a0, 1);
-                                a1 = __funnelshift_l(__float_as_uint(__fsub_rn(z, th)), a1, 1);
-                            }
-                        } else {
-                            if (anyl) {
-#pragma unroll
-                                for (int k = 31; k >= 0; k--)
-                                    a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl, __uint_as_float(v[k]))), a0, 1);
-                            }
-                            if (anyh) {
-#pragma unroll
-                                for (int k = 31; k >= 0; k--)
-                                    a1 = __funnelshift_l(__float_as_uint(__fsub_rn(__uint_as_float(v[k]), th)), a1, 1);
-                            }
-                        }
-                        m0 = nl ? ~a0 : 0u;  // z <= tl
-                        m1 = nh ? ~a1 : 0u;  // z >= th
-                    }
-                    setn(pm, c, m0);
-                    setn(px, c, m1);
-                }
                 float ex_mn[NBK], ex_mx[NBK];
 #pragma unroll
                 for (int bk = 0; bk < NBK; bk++) {
                     ex_mn[bk] = INFINITY;
                     ex_mx[bk] = -INFINITY;
                 }
-                bool pend = (pm[0] | pm[1] | pm[2] | pm[3] | px[0] | px[1] | px[2] | px[3]) != 0;
-                while (__any_sync(0xffffffffu, pend)) {
-                    // every lane's candidates take consecutive slots (warp prefix sum of the
-                    // counts); one cooperative round serves up to kQCap of them
-                    const int cnt = __popc(pm[0] | px[0]) + __popc(pm[1] | px[1]) + __popc(pm[2] | px[2]) +
-                                    __popc(pm[3] | px[3]);
-                    int inc = cnt;
-#pragma unroll
-                    for (int off = 1; off < 32; off <<= 1) {
-                        const int t = __shfl_up_sync(0xffffffffu, inc, off);
-                        if (lane >= off) inc += t;
-                    }
-                    const int base = inc - cnt;
-                    const int total = __shfl_sync(0xffffffffu, inc, 31);
-                    int slot = base;
+                int nj = 0;
+                auto flush = [&]() {
+                    __syncwarp();
+                    run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
+                    __syncwarp();
 #pragma unroll 1
-                    for (int c = 0; c < 4 && slot < kQCap; c++) {
-                        uint32_t m = pickn(pm, c) | pickn(px, c);
-                        while (m && slot < kQCap) {
-                            const uint32_t col = (uint32_t)(c * 32 + __ffs(m) - 1);
-                            qjob[2 * slot] = (uint32_t)row | (col << 8);
-                            m &= m - 1;
-                            slot++;
+                    for (int j = 0; j < nj; j++) {
+                        const uint32_t w = jobs[j];
+                        const float ze = rowbuf[j];
+                        if ((int)(w & 31u) == lane) {
+                            const int bk = (int)((w >> 8) & 127u) / blk;
+                            if (w & 0x10000u) setn(ex_mn, bk, fminf(pickn(ex_mn, bk), ze));
+                            if (w & 0x20000u) setn(ex_mx, bk, fmaxf(pickn(ex_mx, bk), ze));
                         }
                     }
                     __syncwarp();
-                    run_jobs<kJobSlots>(qjob, min(total, kQCap), stg, Gf, g, lane);
-                    __syncwarp();
-                    // the same candidates in the same order: fold the exact values in
-                    slot = base;
+                    nj = 0;
+                };
 #pragma unroll 1
-                    for (int c = 0; c < 4 && slot < kQCap; c++) {
-                        const int bk = c / CPB;
-                        uint32_t cm = pickn(pm, c), cx = pickn(px, c);
-                        uint32_t m = cm | cx;
-                        float emn = pickn(ex_mn, bk), emx = pickn(ex_mx, bk);
-                        while (m && slot < kQCap) {
-                            const uint32_t bit = m & (0u - m);
-                            const float ze = __uint_as_float(qjob[2 * slot + 1]);
-                            if (cm & bit) emn = fminf(emn, ze);
-                            if (cx & bit) emx = fmaxf(emx, ze);
-                            cm &= ~bit;
-                            cx &= ~bit;
-                            m &= m - 1;
-                            slot++;
-                        }
-                        setn(ex_mn, bk, emn);
-                        setn(ex_mx, bk, emx);
-                        setn(pm, c, cm);
-                        setn(px, c, cx);
+                for (int c = 0; c < 4; c++) {
+                    const int bk = c / CPB;
+                    const int need = (amb >> (2 * bk)) & 3;
+                    const float e2 = 2.0f * pickn(E, bk);
+                    float tl = __fadd_rn(pickn(mn, bk), e2), th = __fsub_rn(pickn(mx, bk), e2);
+                    const bool nl = need != 0 && pickn(cmn, c) <= tl;
+                    const bool nh = (need & 1) && pickn(cmx, c) >= th;
+                    uint32_t todo = __ballot_sync(0xffffffffu, nl || nh);
+                    if (todo == 0) continue;
+                    if (!nl) tl = -INFINITY;
+                    if (!nh) th = INFINITY;
+                    uint32_t left = 0xffffffffu;  // values of row src that no earlier round has taken
+                    while (todo) {
+                        uint32_t v[32];
+                        tmem_ld32(tacc + c * 32, v);
+                        tmem_wait_ld();
+                        do {
+                            const int src = __ffs(todo) - 1;
+                            const float stl = __shfl_sync(0xffffffffu, tl, src), sth = __shfl_sync(0xffffffffu, th, src);
+                            const float z = spread(v, src);
+                            const uint32_t job = (uint32_t)(q4 * 32 + src) | (uint32_t)(c * 32 + lane) << 8 |
+                                                 (z <= stl ? 0x10000u : 0u) | (z >= sth ? 0x20000u : 0u);
+                            left = append(__ballot_sync(0xffffffffu, (job & 0x30000u) != 0u) & left, job, nj);
+                            if (left) break;  // the list is full
+                            todo &= todo - 1;
+                            left = 0xffffffffu;
+                        } while (todo);
+                        if (todo) flush();  // (the row's values need not survive it: they are loaded again)
                     }
-                    __syncwarp();
-                    pend = (pm[0] | pm[1] | pm[2] | pm[3] | px[0] | px[1] | px[2] | px[3]) != 0;
                 }
+                if (nj) flush();
 #pragma unroll
                 for (int bk = 0; bk < NBK; bk++) {
                     const int need = (amb >> (2 * bk)) & 3;
@@ -639,13 +619,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     // every code is the exact rule's)
                     lim[bk] = !TILE && mu < 0.99e-4f ? 2.0f : 0.5f - mu;
                     const float tlo = (mn[bk] - E[bk]) * r + cc, thi = (mx[bk] + E[bk]) * r + cc;
-                    fast[bk] = tlo > -0.49f + mu && thi < qmaxf + 0.49f - mu && (TILE || lim[bk] > 1.0f);
+                    fast[bk] = tlo > -0.49f + mu && thi < qmaxf + 0.49f - mu && (kTrack || lim[bk] > 1.0f);
                 }
             }
 
             // ---- 6. codes from z~, stored straight from registers
             uint8_t* crow = a.codes + a.cmap.at(ti.l, ti.s, ti.b, ti.h, ti.t0 + row);
-            uint32_t am[4] = {0, 0, 0, 0};  // values within mu of a rounding boundary
+            int nj = 0;  // values within mu of a rounding boundary, to be recomputed exactly and patched
+            auto patch = [&]() {
+                __syncwarp();
+                run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
+                __syncwarp();
+#pragma unroll 1
+                for (int j = 0; j < nj; j++) {
+                    const uint32_t w = jobs[j];
+                    const float ze = rowbuf[j];
+                    if ((int)(w & 31u) == lane) {
+                        const int col = (int)((w >> 8) & 127u), bk = col / blk;
+                        patch_code<BITS>(crow, col * BITS, quant_code(ze, h2f_bits(pickn(s16, bk)), h2f_bits(pickn(m16, bk)), qmax));
+                    }
+                }
+                __syncwarp();
+                nj = 0;
+            };
 #pragma unroll 1
             for (int c = 0; c < 4; c++) {
                 uint32_t v[32];
@@ -657,58 +653,36 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                 uint32_t words[BITS];
 #pragma unroll
                 for (int w = 0; w < BITS; w++) words[w] = 0;
-                uint32_t mk = 0;
+                float worst = 0.0f;  // the largest distance from an integer of this lane's values
+                const float2 r2 = make_float2(r, r), c2 = make_float2(cz, cz), m2 = make_float2(kMagic, kMagic);
+                const float2 n2 = make_float2(-kMagic, -kMagic);
                 if (__all_sync(0xffffffffu, TILE ? fst || !valid : fst)) {
                     // the same fma and add per value, two values per instruction
-                    const float2 r2 = make_float2(r, r), c2 = make_float2(cz, cz), m2 = make_float2(kMagic, kMagic);
-                    if constexpr (!TILE) {
 #pragma unroll
-                        for (int k = 0; k < 32; k += 2) {
-                            const float2 y = __fadd2_rn(
-                                __ffma2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), r2, c2), m2);
-                            put_code<BITS>(words, k, __float_as_uint(y.x));
-                            put_code<BITS>(words, k + 1, __float_as_uint(y.y));
-                        }
-                    } else {
-                        // the largest distance from an integer decides whether the chunk holds a value
-                        // near a rounding boundary at all; only then are the values marked one by one
-                        const float lm = pickn(lim, bk);
-                        float worst = 0.0f;
-                        const float2 n2 = make_float2(-kMagic, -kMagic);
-#pragma unroll
-                        for (int k = 0; k < 32; k += 2) {
-                            const float2 t =
-                                __ffma2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), r2, c2);
-                            const float2 y = __fadd2_rn(t, m2);
-                            put_code<BITS>(words, k, __float_as_uint(y.x));
-                            put_code<BITS>(words, k + 1, __float_as_uint(y.y));
+                    for (int k = 0; k < 32; k += 2) {
+                        const float2 t = __ffma2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), r2, c2);
+                        const float2 y = __fadd2_rn(t, m2);
+                        put_code<BITS>(words, k, __float_as_uint(y.x));
+                        put_code<BITS>(words, k + 1, __float_as_uint(y.y));
+                        if constexpr (kTrack) {
                             const float2 q = __fadd2_rn(y, n2);
-                            const float2 e = __fadd2_rn(t, make_float2(-q.x, -q.y));
+                            const float2 e = __ffma2_rn(q, make_float2(-1.0f, -1.0f), t);  // exact
                             worst = max3f(worst, fabsf(e.x), fabsf(e.y));
-                        }
-                        if (__any_sync(0xffffffffu, worst > lm)) {
-                            tmem_ld32(tacc + c * 32, v);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int k = 31; k >= 0; k--) {
-                                const float t = fmaf(__uint_as_float(v[k]), r, cz);
-                                const float y = t + kMagic;
-                                mk = __funnelshift_l(__float_as_uint(__fsub_rn(lm, fabsf(t - (y - kMagic)))), mk, 1);
-                            }
                         }
                     }
                 } else {
                     // clamping before the rounding gives the same code as clamping after it
-                    const float lm = pickn(lim, bk);
 #pragma unroll
-                    for (int k = 31; k >= 0; k--) {
-                        float t = fmaf(__uint_as_float(v[k]), r, cz);
-                        t = fminf(fmaxf(t, 0.0f), qmaxf);
-                        const float y = t + kMagic;
-                        mk = __funnelshift_l(__float_as_uint(__fsub_rn(lm, fabsf(t - (y - kMagic)))), mk, 1);
-                        put_code<BITS>(words, k, __float_as_uint(y));
+                    for (int k = 0; k < 32; k += 2) {
+                        float2 t = __ffma2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), r2, c2);
+                        t = make_float2(fminf(fmaxf(t.x, 0.0f), qmaxf), fminf(fmaxf(t.y, 0.0f), qmaxf));
+                        const float2 y = __fadd2_rn(t, m2);
+                        put_code<BITS>(words, k, __float_as_uint(y.x));
+                        put_code<BITS>(words, k + 1, __float_as_uint(y.y));
+                        const float2 q = __fadd2_rn(y, n2);
+                        const float2 e = __ffma2_rn(q, make_float2(-1.0f, -1.0f), t);  // exact
+                        worst = max3f(worst, fabsf(e.x), fabsf(e.y));
                     }
-                    if (!TILE && fst) mk = 0;
                 }
 #pragma unroll
                 for (int w = 0; w < BITS; w++) words[w] -= pack_bias<BITS>(w);
@@ -726,54 +700,30 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
 #pragma unroll
                         for (int w = 0; w < BITS; w++) dst[w] = words[w];
                     }
-                    setn(am, c, mk);
+                }
+                // ---- 7. values within mu of a rounding boundary: exact recompute and patch
+                const float lm = pickn(lim, bk);
+                uint32_t todo = __ballot_sync(0xffffffffu, valid && worst > lm);
+                uint32_t left = 0xffffffffu;
+                while (todo) {
+                    tmem_ld32(tacc + c * 32, v);
+                    tmem_wait_ld();
+                    do {
+                        const int src = __ffs(todo) - 1;
+                        const float sr = __shfl_sync(0xffffffffu, r, src), sc = __shfl_sync(0xffffffffu, cz, src);
+                        const float sl = __shfl_sync(0xffffffffu, lm, src);
+                        const float z = spread(v, src);
+                        const float t = fminf(fmaxf(fmaf(z, sr, sc), 0.0f), qmaxf);
+                        left = append(__ballot_sync(0xffffffffu, fabsf(t - ((t + kMagic) - kMagic)) > sl) & left,
+                                      (uint32_t)(q4 * 32 + src) | (uint32_t)(c * 32 + lane) << 8, nj);
+                        if (left) break;  // the list is full
+                        todo &= todo - 1;
+                        left = 0xffffffffu;
+                    } while (todo);
+                    if (todo) patch();
                 }
             }
-
-            // ---- 7. values within mu of a rounding boundary: exact recompute and patch
-            bool pend = (am[0] | am[1] | am[2] | am[3]) != 0;
-            while (__any_sync(0xffffffffu, pend)) {
-                const int cnt = __popc(am[0]) + __popc(am[1]) + __popc(am[2]) + __popc(am[3]);
-                int inc = cnt;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, inc, off);
-                    if (lane >= off) inc += t;
-                }
-                const int base = inc - cnt;
-                const int total = __shfl_sync(0xffffffffu, inc, 31);
-                int slot = base;
-#pragma unroll 1
-                for (int c = 0; c < 4 && slot < kQCap; c++) {
-                    uint32_t m = pickn(am, c);
-                    while (m && slot < kQCap) {
-                        const uint32_t col = (uint32_t)(c * 32 + __ffs(m) - 1);
-                        qjob[2 * slot] = (uint32_t)row | (col << 8);
-                        m &= m - 1;
-                        slot++;
-                    }
-                }
-                __syncwarp();
-                run_jobs<kJobSlots>(qjob, min(total, kQCap), stg, Gf, g, lane);
-                __syncwarp();
-                slot = base;
-#pragma unroll 1
-                for (int c = 0; c < 4 && slot < kQCap; c++) {
-                    const int bk = c / CPB;
-                    uint32_t m = pickn(am, c);
-                    const float sb = h2f_bits(pickn(s16, bk)), mb = h2f_bits(pickn(m16, bk));
-                    while (m && slot < kQCap) {
-                        const int col = c * 32 + __ffs(m) - 1;
-                        const float ze = __uint_as_float(qjob[2 * slot + 1]);
-                        patch_code<BITS>(crow, col * BITS, quant_code(ze, sb, mb, qmax));
-                        m &= m - 1;
-                        slot++;
-                    }
-                    setn(am, c, m);
-                }
-                __syncwarp();
-                pend = (am[0] | am[1] | am[2] | am[3]) != 0;
-            }
+            if (nj) patch();
 
             // ---- 8. scales (tiles: one set for the 16 rows); release the stage and the accumulator
             if (valid && (!TILE || (row & (CG_TILE_TOKENS - 1)) == 0)) {
