@@ -231,7 +231,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
     const tc::Sched& S = P.S;
     const int g = a.g, npass = kNPass;
     constexpr int blk = kD / NBK;  // quantization block: NBK blocks per row
-    const int gb = g < 16 ? 16 : g;
     constexpr int nbk = NBK;
     // values per lane and memory round trip in the exact recompute (measured: 4 with two
     // blocks per row, the 8B-shaped cache; 2 with one or four)
@@ -309,8 +308,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0 && my_tiles > 0) {
-            const uint32_t idesc = idesc_bf16_f32(128, KEYS ? 128 : gb);
-            const int kg = KEYS ? 128 : gb;  // keys: one chain over the full K
+            static_assert(KEYS, "rows are encoded by tc_rows_encode_kernel");
+            constexpr uint32_t idesc = idesc_bf16_f32(128, 128);  // keys: one chain over the full K
             int64_t cur = -1;
             int committed = 0;
             tc::TileIter it;
@@ -331,25 +330,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                     break;
                 }
                 tc_fence_after();
-                const uint32_t a_base = smem_u32(stages + st * kTileBytes);
+                // D[channel][token] = G x^T: the operands' K-steps lie at constant offsets, so the single
+                // issuing thread spends two adds per MMA. Descriptors built in the loop cost 1 % (three
+                // bit keys of the 8B-shaped cache, with their values: 4.52 -> 4.48 ms)
+                const uint64_t gdesc = sdesc_sw128(smem_u32(bsplit)), xdesc = sdesc_sw128(smem_u32(stages + st * kTileBytes));
                 const uint32_t d_base = tmem + buf * 128;
-                for (int p = 0; p < npass; p++) {
-                    const uint32_t b_base = smem_u32(bsplit) + p * bsz;
-                    for (int r = 0; r < 128 / kg; r++) {
-                        for (int ks = 0; ks < kg / 16; ks++) {
-                            const int k0 = r * kg + ks * 16;
-                            const uint32_t a_addr = a_base + (k0 >> 6) * 16384 + (k0 & 63) * 2;
-                            const uint32_t b_addr = b_base + (fullk ? (k0 >> 6) * 16384 : 0) +
-                                                    (KEYS ? 0 : (r * gb) * 128) + (k0 & 63) * 2;
-                            if (KEYS)  // D[channel][token] = G x^T
-                                mma_bf16(d_base, sdesc_sw128(b_addr), sdesc_sw128(a_addr), idesc,
-                                         (p > 0 || ks > 0) ? 1u : 0u);
-                            else  // D[token][channel] = x G^T, one chain per gauge group
-                                mma_bf16(d_base + r * gb, sdesc_sw128(a_addr), sdesc_sw128(b_addr), idesc,
-                                         (p > 0 || ks > 0) ? 1u : 0u);
-                        }
+#pragma unroll
+                for (int p = 0; p < kNPass; p++)
+#pragma unroll
+                    for (int ks = 0; ks < kD / 16; ks++) {
+                        const uint32_t off = (uint32_t)((ks >> 2) * 16384 + (ks & 3) * 32) >> 4;
+                        mma_bf16(d_base, gdesc + (uint32_t)(p * 32768 >> 4) + off, xdesc + off, idesc, (p > 0 || ks > 0) ? 1u : 0u);
                     }
-                }
                 mma_commit(&M->accfull[buf]);
                 const bool last_of_seg = (i + 1 == my_tiles) || it.seg_last(a);
                 if (last_of_seg) mma_commit(&M->bfree);
