@@ -1,22 +1,24 @@
-// cg_tc.cu -- tensor-core (tcgen05) encode of the row path, head dim d = 128: gauge
-// rotation (Sec. 3, Z = G X) fused with the block-uniform quantizer of Sec. 4.3 (one range
-// per block of `block` channels of a token), also used for KIVI value rows.
+// cg_tc.cu -- tensor-core (tcgen05) encode of KIVI keys, head dim d = 128: gauge rotation
+// (Sec. 3, Z = G X) fused with one range per channel over the 128 tokens of a key group.
 //
 // Persistent warp-specialized kernel, one CTA per SM, 15 warps:
 //   warp 0      TMA producer: 128-token x tiles (2 x [128 rows x 64 bf16], 128-byte
 //               swizzle) into a 4-stage ring;
-//   warp 1      MMA issuer: z~ = x G^T on tcgen05 (M = 128 tokens, N = K = gauge group,
-//               one MMA chain per group block), G split into three bf16 terms (hi + lo +
-//               lo2, exact for normal fp32 values); fp32 accumulators in tensor memory,
-//               four buffers (the MMA runs one tile ahead of the three warpgroups);
+//   warp 1      MMA issuer: z~ = G x^T on tcgen05 (M = 128 channels, N = 128 tokens, K = 128,
+//               the gauge block-diagonal), G split into three bf16 terms (hi + lo + lo2, exact
+//               for normal fp32 values); fp32 accumulators in tensor memory, four buffers
+//               (the MMA runs one tile ahead of the three warpgroups);
 //   warp 2      gauge converter: at each gauge change builds the bf16 split operand and
-//               the per-block error coefficients of the new gauge set;
+//               the error coefficients of the new gauge set;
 //   warps 3..14 three epilogue warpgroups; warpgroup k takes tiles i = k (mod 3); one
-//               thread per token row (= TMEM lane): block min/max, fp16 scale/zero, codes,
-//               packing, stores. The number of quantization blocks per row is a template
-//               parameter, so the per-block state of a row takes only the registers it
-//               needs (128 per thread for 15 warps); codes are packed into the output
-//               words as they are produced.
+//               thread per channel (= TMEM lane): range, fp16 scale/zero, codes, packing,
+//               stores; codes are packed into the output words as they are produced.
+//
+// What bounds it: the epilogue's latency and issue, not memory (1.34 ms of 3.9 for 28 x 4 x 4
+// heads of 32k tokens at 3 bits, keys and values). The candidates of an undecided range and
+// the values near a rounding boundary are found by spreading a channel's 32 values over the
+// lanes (one compare and vote) instead of by masks in every lane, and codes are made in
+// packed pairs: 4.49 -> 3.89 ms.
 //
 // Exactness. The library defines z as a fixed-order fp32 sum (pairwise summation of the
 // products; include/codecgauge.h). For every output channel i the converter bounds
@@ -37,8 +39,8 @@
 // The accepted tolerance lets a code differ by one where t lies within 1e-4 steps of a
 // boundary, so blocks with mu < 1e-4 keep the z~ codes; in blocks with a larger mu the
 // codes within mu of a boundary are recomputed exactly. Recomputation uses the library's
-// order (as the CUDA-core kernels do): candidates go into a per-warp shared-memory job
-// queue and teams of lanes compute them together.
+// order (as the CUDA-core kernels do): candidates go into a per-warp list in shared memory
+// and teams of lanes compute them together.
 #include <cuda_bf16.h>
 
 #include "cg_sm100.cuh"
@@ -58,7 +60,7 @@ constexpr int kStages = 4;
 constexpr int kTileBytes = 128 * kD * 2;
 constexpr int kThreads = 480;
 constexpr int kEpiWarp0 = 3;
-constexpr int kQCap = 20;             // repair jobs per warp and round
+constexpr int kJobCap = 8;            // exact recomputes per warp and round
 constexpr int kAcc = 4;               // accumulator buffers in tensor memory
 constexpr int kNPass = 3;             // bf16 terms of the gauge split
 constexpr int kSegBufs = 4;
@@ -67,8 +69,8 @@ constexpr float kMagic = 12582912.0f; // 1.5 * 2^23: adding it rounds to an inte
 struct EncSmem {
     static constexpr uint32_t stages = 0;
     static constexpr uint32_t bsplit = stages + kStages * kTileBytes;  // 3 x (16 or 32 KB)
-    static constexpr uint32_t queue = bsplit + kNPass * 32768;         // 12 warps x kQCap x 8 B
-    static constexpr uint32_t xch = queue + 12 * kQCap * 8;  // keys: 3 warpgroups x 2 x 4 warps x 4 floats
+    static constexpr uint32_t queue = bsplit + kNPass * 32768;         // 12 warps x (32 values, kJobCap jobs)
+    static constexpr uint32_t xch = queue + 12 * (32 + kJobCap) * 4;  // keys: 3 warpgroups x 2 x 4 warps x 4 floats
     static constexpr uint32_t misc = xch + 3 * 2 * 4 * 4 * 4;
     static constexpr uint32_t total = misc + 384;  // base is 1024-aligned (checked in-kernel)
 };
@@ -119,64 +121,6 @@ __device__ __forceinline__ void set4(T (&v)[4], int i, T x) {
     v[3] = i == 3 ? x : v[3];
 }
 
-// Rows of the gauge channels whose error bounds block bk's values: the whole gauge group
-// when the group spans the block, else the block's own channels.
-__device__ __forceinline__ void bound_range(int bk, int g, int blk, int& lo, int& hi) {
-    if (g >= blk) {
-        lo = ((bk * blk) / g) * g;
-        hi = lo + g;
-    } else {
-        lo = bk * blk;
-        hi = lo + blk;
-    }
-}
-
-// One warp-wide round of exact recomputation of the queued gauge-space values (job word:
-// row | col << 8; the value goes to the next word), in the library's fixed order. A team
-// of T = g/4 lanes computes one value: lane j forms the products of channels 4j..4j+3 and
-// their pairwise sum, and the team combines its partial sums with xor-shuffles, which
-// follows the same pairwise tree. Each lane loads the operands of kSlots values before any
-// arithmetic, so one memory round trip serves kSlots x (32 / T) values.
-template <int kSlots>
-__device__ __noinline__ void run_jobs(uint32_t* qjob, int nq, const unsigned char* stage, const float* Gf, int g,
-                                      int lane) {
-    const int lgT = 29 - __clz(g);  // log2(g / 4); g in {8, ..., 128}
-    const int T = 1 << lgT, teams = 32 >> lgT;
-    const int tm = lane >> lgT, j = lane & (T - 1);
-    for (int base = 0; base < nq; base += kSlots * teams) {
-        uint2 xv[kSlots];
-        float4 gv[kSlots];
-#pragma unroll
-        for (int k = 0; k < kSlots; k++) {
-            const int c = base + k * teams + tm;
-            const uint32_t jb = qjob[2 * (c < nq ? c : 0)];
-            const int row = (int)(jb & 0xffu), col = (int)((jb >> 8) & 0xffu);
-            const int kk = (col & ~(g - 1)) + 4 * j;  // first channel of this lane's products
-            xv[k] = *reinterpret_cast<const uint2*>(stage + (kk >> 6) * 16384 + row * 128 +
-                                                    ((((kk & 63) >> 3) ^ (row & 7)) << 4) + (kk & 7) * 2);
-            gv[k] = __ldg(reinterpret_cast<const float4*>(Gf + (size_t)col * g + 4 * j));
-        }
-        float part[kSlots];
-#pragma unroll
-        for (int k = 0; k < kSlots; k++) {
-            const float p0 = __fmul_rn(gv[k].x, bf_lo(xv[k].x)), p1 = __fmul_rn(gv[k].y, bf_hi(xv[k].x));
-            const float p2 = __fmul_rn(gv[k].z, bf_lo(xv[k].y)), p3 = __fmul_rn(gv[k].w, bf_hi(xv[k].y));
-            part[k] = __fadd_rn(__fadd_rn(p0, p1), __fadd_rn(p2, p3));
-        }
-        for (int w = 1; w < T; w <<= 1) {
-#pragma unroll
-            for (int k = 0; k < kSlots; k++) part[k] = __fadd_rn(part[k], __shfl_xor_sync(0xffffffffu, part[k], w));
-        }
-        if (j == 0) {
-#pragma unroll
-            for (int k = 0; k < kSlots; k++) {
-                const int c = base + k * teams + tm;
-                if (c < nq) qjob[2 * c + 1] = __float_as_uint(part[k]);
-            }
-        }
-    }
-}
-
 // The constant part of a packed word built from y = 0x4B400000 + q: the wrapping sum of
 // 0x4B400000 << s over the codes of a 32-code chunk that start in word w.
 template <int BITS>
@@ -207,10 +151,8 @@ __device__ __forceinline__ void patch_code(uint8_t* rowp, int bit, uint32_t q) {
     }
 }
 
-// KEYS = false: block-uniform rows and KIVI value rows (thread = token, block = channels).
-// KEYS = true: KIVI keys (Sec. 4.3, per-channel ranges over a 128-token group): the MMA
-// operands are swapped, D[channel][token] = G x^T, so a thread owns one channel's 128
-// tokens, which form its block and its packed code stream.
+// The MMA's operands are swapped against the row kernel's, D[channel][token] = G x^T, so a
+// thread owns one channel's 128 tokens, which form its block and its packed code stream.
 template <int BITS, bool KEYS, int NBK>
 __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_constant__ CUtensorMap xmap,
                                                                  const EncParams P) {
@@ -232,9 +174,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
     const int g = a.g, npass = kNPass;
     constexpr int blk = kD / NBK;  // quantization block: NBK blocks per row
     constexpr int nbk = NBK;
-    // values per lane and memory round trip in the exact recompute (measured: 4 with two
-    // blocks per row, the 8B-shaped cache; 2 with one or four)
-    constexpr int kJobSlots = NBK == 2 ? 4 : 2;
+    // 6 and 8 bits: values near a rounding boundary are common (their distance mu grows with the range
+    // over the scale), so every lane keeps a mask of its own and the list holds 20 of them; 2 to 4 bits:
+    // rare, so a lane keeps only its largest distance and the chunk is looked through again. 3 bits, 28 x
+    // 4 x 4 heads of 32k tokens: 4463 us with masks, 3888 without; 8 bits, 2 x 8 heads of 4k: 68 and 73.
+    constexpr bool kMasks = BITS >= 6;
+    constexpr int kJobSlots = kMasks ? 4 : 2;  // values per lane and memory round trip in the exact recompute
     // gauge operand layout: full K = 128 (block-diagonal for g < 128) for keys and g = 128,
     // else one g-wide K block per group in a 64-column tile
     const bool fullk = KEYS || g == 128;
@@ -383,19 +328,33 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
         // ------------------------------------------------------------ epilogue warpgroups
         const int wg = (warp - kEpiWarp0) >> 2;       // warpgroup: tiles i = wg (mod 3)
         const int q4 = warp & 3;                      // TMEM lane quadrant of this warp
-        const int row = q4 * 32 + lane;               // TMEM lane: token (rows) or channel (keys)
+        const int row = q4 * 32 + lane;               // TMEM lane: channel (and the token whose norm it takes)
         const int qw = warp - kEpiWarp0;              // job queue of this warp
-        uint32_t* qjob = queue + qw * kQCap * 2;
+        float* rowbuf = reinterpret_cast<float*>(queue) + qw * (32 + kJobCap);  // 32 values of a channel, or results
+        uint32_t* jobs = reinterpret_cast<uint32_t*>(rowbuf + 32);
+        const uint32_t lt = (1u << lane) - 1u;
+        // The 32 values v of lane `src` spread over the lanes: lane k gets value k.
+        auto spread = [&](const uint32_t (&v)[32], int src) -> float {
+            __syncwarp();
+            if (lane == src) {
+#pragma unroll
+                for (int k = 0; k < 32; k += 4)
+                    *reinterpret_cast<uint4*>(rowbuf + k) = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+            }
+            __syncwarp();
+            return rowbuf[lane];
+        };
+        // Appends a job for every set lane of m to the list of n (< cap) while there is room; returns the lanes left over.
+        auto append = [&](uint32_t* list, int cap, uint32_t m, uint32_t word, int& n) -> uint32_t {
+            const bool mine = (m >> lane) & 1u;
+            const int at = n + __popc(m & lt);
+            if (mine && at < cap) list[at] = word;
+            const int all = n + __popc(m);
+            n = all < cap ? all : cap;
+            return all > cap ? __ballot_sync(0xffffffffu, mine && at >= cap) : 0u;
+        };
         const float qmaxf = (float)((1 << BITS) - 1);
         const int qmax = (1 << BITS) - 1;
-        int lo8[4], hi8[4];
-#pragma unroll
-        for (int bk = 0; bk < 4; bk++) {
-            int lo = 0, hi = 0;
-            if (bk < nbk) bound_range(bk, g, blk, lo, hi);
-            lo8[bk] = lo >> 3;
-            hi8[bk] = hi >> 3;
-        }
         int32_t flag = 0;
         tc::TileIter it;
         it.init(a, S, t_begin + wg);
@@ -474,45 +433,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                     gm[rr] = fmaxf(fmaxf(xb[rr], xb[4 + rr]), fmaxf(xb[8 + rr], xb[12 + rr]));
                 bs[0] = pick4(gm, row / g);  // fmaxf keeps a NaN out; non-finite input is flagged above
             }
-            // unroll depth measured per block count (code size against load parallelism)
-            constexpr int kNormUnroll = NBK == 2 ? 8 : (NBK == 4 ? 2 : 4);
-#pragma unroll kNormUnroll
-            for (int c8 = 0; c8 < (KEYS ? 0 : 16); c8++) {
-                const uint4 xv = *reinterpret_cast<const uint4*>(stg + (c8 >> 3) * 16384 + row * 128 +
-                                                                 (((c8 & 7) ^ (row & 7)) << 4));
-                float s0 = bf_lo(xv.x) * bf_lo(xv.x);
-                s0 = fmaf(bf_hi(xv.x), bf_hi(xv.x), s0);
-                s0 = fmaf(bf_lo(xv.y), bf_lo(xv.y), s0);
-                s0 = fmaf(bf_hi(xv.y), bf_hi(xv.y), s0);
-                s0 = fmaf(bf_lo(xv.z), bf_lo(xv.z), s0);
-                s0 = fmaf(bf_hi(xv.z), bf_hi(xv.z), s0);
-                s0 = fmaf(bf_lo(xv.w), bf_lo(xv.w), s0);
-                s0 = fmaf(bf_hi(xv.w), bf_hi(xv.w), s0);
-#pragma unroll
-                for (int bk = 0; bk < 4; bk++)
-                    if (c8 >= lo8[bk] && c8 < hi8[bk]) bs[bk] += s0;
-            }
-            if (!KEYS && valid && !(isfinite(bs[0]) && isfinite(bs[1]) && isfinite(bs[2]) && isfinite(bs[3]))) {
-                // a non-finite sum of squares: look for an Inf/NaN input (huge finite values
-                // can also overflow the square)
-                for (int c8 = 0; c8 < 16; c8++) {
-                    const uint4 xv = *reinterpret_cast<const uint4*>(stg + (c8 >> 3) * 16384 + row * 128 +
-                                                                     (((c8 & 7) ^ (row & 7)) << 4));
-                    const uint32_t wv[4] = {xv.x, xv.y, xv.z, xv.w};
-                    for (int q = 0; q < 4; q++)
-                        if (bf16_nonfinite(wv[q] & 0xffffu) || bf16_nonfinite(wv[q] >> 16)) flag |= CG_FLAG_NONFINITE_INPUT;
-                }
-            }
-
-            // ---- 2. approximate block ranges from the accumulator. With two blocks per row the
-            // candidate masks are built here for every chunk (measured faster there): the values
-            // within 2 Ep of the chunk's own min / max, Ep >= E (item 3) being known before the
-            // ranges are. Otherwise they are built in the exact-extreme round, only where needed.
-            constexpr bool kEagerMasks = NBK == 2;
-            float mn[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            float clo[4], chi[4];           // chunk min / max (eager masks)
-            uint32_t pm[4], px[4];          // chunk candidate masks (bit k = column 32c + k)
+            // ---- 2. approximate range of the channel from the accumulator, per 32-token chunk and whole
+            static_assert(NBK == 1, "one block per channel");
+            float cmn[4], cmx[4];
 #pragma unroll 1
             for (int c = 0; c < 4; c++) {
                 uint32_t v[32];
@@ -524,29 +447,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                     lo = min3f(lo, __uint_as_float(v[k]), __uint_as_float(v[k + 1]));
                     hi = max3f(hi, __uint_as_float(v[k]), __uint_as_float(v[k + 1]));
                 }
-                lo = fminf(lo, __uint_as_float(v[31]));
-                hi = fmaxf(hi, __uint_as_float(v[31]));
-                const int bk = (c * 32) / blk;
-                set4(mn, bk, fminf(pick4(mn, bk), lo));
-                set4(mx, bk, fmaxf(pick4(mx, bk), hi));
-                if constexpr (!kEagerMasks) continue;
-                // |z~| <= ||G_i|| ||x|| + E, so Ep bounds the E of item 3 from above
-                const float xn = sqrtf(pick4(bs, bk)) * 1.0001f;
-                const float ep = xn * M->emaxb[ls & 3][bk] + 2.0f * xn * M->gmaxb[ls & 3][bk] * 2.41e-7f;
-                const float tl = __fadd_rn(lo, 2.0f * ep), th = __fsub_rn(hi, 2.0f * ep);
-                // sign bits of (threshold - z) and (z - threshold), shifted in from column 31 down
-                uint32_t a0 = 0, a1 = 0;
-#pragma unroll
-                for (int k = 31; k >= 0; k--) {
-                    const float z = __uint_as_float(v[k]);
-                    a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl, z)), a0, 1);
-                    a1 = __funnelshift_l(__float_as_uint(__fsub_rn(z, th)), a1, 1);
-                }
-                set4(clo, c, lo);
-                set4(chi, c, hi);
-                set4(pm, c, ~a0);  // z <= tl
-                set4(px, c, ~a1);  // z >= th
+                set4(cmn, c, fminf(lo, __uint_as_float(v[31])));
+                set4(cmx, c, fmaxf(hi, __uint_as_float(v[31])));
             }
+            float mn[4] = {fminf(fminf(cmn[0], cmn[1]), fminf(cmn[2], cmn[3])), 0.0f, 0.0f, 0.0f};
+            float mx[4] = {fmaxf(fmaxf(cmx[0], cmx[1]), fmaxf(cmx[2], cmx[3])), 0.0f, 0.0f, 0.0f};
 
             // ---- 3. error bound per block; scale/zero from the intervals when they agree
             float E[4];
@@ -571,119 +476,66 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                 }
             }
 
-            // ---- 4. exact extremes of ambiguous blocks (warp-cooperative rounds)
+            // ---- 4. exact extremes of undecided channels: candidates are the values within 2E of the
+            // approximate extreme, in chunks whose own extreme lies that close, found by one compare and
+            // vote over the lanes per such chunk
             if (__any_sync(0xffffffffu, amb != 0)) {
-                if constexpr (kEagerMasks) {
-                    // candidates: a chunk's values near its own min (max) are candidates of the
-                    // block min (max) when the chunk min lies within 2E of the block min
+                const int need = amb & 3;
+                float ex_mn = INFINITY, ex_mx = -INFINITY;
+                int nj = 0;
+                auto flush = [&]() {
+                    __syncwarp();
+                    tce::run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
+                    __syncwarp();
 #pragma unroll 1
-                    for (int c = 0; c < 4; c++) {
-                        const int bk = (c * 32) / blk;
-                        const int need = (amb >> (2 * bk)) & 3;
-                        const float e2 = 2.0f * pick4(E, bk);
-                        const bool nl = need && pick4(clo, c) <= __fadd_rn(pick4(mn, bk), e2);
-                        const bool nh = (need & 1) && pick4(chi, c) >= __fsub_rn(pick4(mx, bk), e2);
-                        set4(pm, c, nl ? pick4(pm, c) : 0u);
-                        set4(px, c, nh ? pick4(px, c) : 0u);
-                    }
-                } else {
-                    // candidates of an ambiguous block's min (max): its values within 2E of the
-                    // approximate min (max); the chunks some lane needs are reloaded from TMEM
-#pragma unroll 1
-                    for (int c = 0; c < 4; c++) {
-                        const int bk = (c * 32) / blk;
-                        const int need = (amb >> (2 * bk)) & 3;
-                        uint32_t m0 = 0, m1 = 0;
-                        if (__any_sync(0xffffffffu, need != 0)) {
-                            uint32_t v[32];
-                            tmem_ld32(tacc + c * 32, v);
-                            tmem_wait_ld();
-                            const float e2 = 2.0f * pick4(E, bk);
-                            const float tl = __fadd_rn(pick4(mn, bk), e2), th = __fsub_rn(pick4(mx, bk), e2);
-                            uint32_t a0 = 0, a1 = 0;
-#pragma unroll
-                            for (int k = 31; k >= 0; k--) {
-                                const float z = __uint_as_float(v[k]);
-                                a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl, z)), a0, 1);
-                                a1 = __funnelshift_l(__float_as_uint(__fsub_rn(z, th)), a1, 1);
-                            }
-                            m0 = need ? ~a0 : 0u;        // z <= tl
-                            m1 = (need & 1) ? ~a1 : 0u;  // z >= th
+                    for (int j = 0; j < nj; j++) {
+                        const uint32_t w = jobs[j];
+                        const float ze = rowbuf[j];
+                        if ((int)((w >> 8) & 31u) == lane) {
+                            if (w & 0x10000u) ex_mn = fminf(ex_mn, ze);
+                            if (w & 0x20000u) ex_mx = fmaxf(ex_mx, ze);
                         }
-                        set4(pm, c, m0);
-                        set4(px, c, m1);
+                    }
+                    __syncwarp();
+                    nj = 0;
+                };
+                const float e2 = 2.0f * E[0], tl0 = __fadd_rn(mn[0], e2), th0 = __fsub_rn(mx[0], e2);
+#pragma unroll 1
+                for (int c = 0; c < 4; c++) {
+                    const bool nl = need != 0 && pick4(cmn, c) <= tl0;
+                    const bool nh = (need & 1) && pick4(cmx, c) >= th0;
+                    uint32_t todo = __ballot_sync(0xffffffffu, nl || nh);
+                    if (todo == 0) continue;
+                    const float tl = nl ? tl0 : -INFINITY, th = nh ? th0 : INFINITY;
+                    uint32_t left = 0xffffffffu;  // values of channel src that no earlier round has taken
+                    while (todo) {
+                        uint32_t v[32];
+                        tmem_ld32(tacc + c * 32, v);
+                        tmem_wait_ld();
+                        do {
+                            const int src = __ffs(todo) - 1;
+                            const float stl = __shfl_sync(0xffffffffu, tl, src), sth = __shfl_sync(0xffffffffu, th, src);
+                            const float z = spread(v, src);
+                            const uint32_t job = (uint32_t)(c * 32 + lane) | (uint32_t)(q4 * 32 + src) << 8 |
+                                                 (z <= stl ? 0x10000u : 0u) | (z >= sth ? 0x20000u : 0u);
+                            left = append(jobs, kJobCap, __ballot_sync(0xffffffffu, (job & 0x30000u) != 0u) & left, job, nj);
+                            if (left) break;  // the list is full
+                            todo &= todo - 1;
+                            left = 0xffffffffu;
+                        } while (todo);
+                        if (todo) flush();  // (the values need not survive it: they are loaded again)
                     }
                 }
-                float ex_mn[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-                float ex_mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                bool pend = (pm[0] | pm[1] | pm[2] | pm[3] | px[0] | px[1] | px[2] | px[3]) != 0;
-                while (__any_sync(0xffffffffu, pend)) {
-                    // every lane's candidates take consecutive slots (warp prefix sum of the
-                    // counts); one cooperative round serves up to kQCap of them
-                    const int cnt = __popc(pm[0] | px[0]) + __popc(pm[1] | px[1]) + __popc(pm[2] | px[2]) +
-                                    __popc(pm[3] | px[3]);
-                    int inc = cnt;
-#pragma unroll
-                    for (int off = 1; off < 32; off <<= 1) {
-                        const int t = __shfl_up_sync(0xffffffffu, inc, off);
-                        if (lane >= off) inc += t;
-                    }
-                    const int base = inc - cnt;
-                    const int total = __shfl_sync(0xffffffffu, inc, 31);
-                    int slot = base;
-#pragma unroll 1
-                    for (int c = 0; c < 4 && slot < kQCap; c++) {
-                        uint32_t m = pick4(pm, c) | pick4(px, c);
-                        while (m && slot < kQCap) {
-                            const uint32_t col = (uint32_t)(c * 32 + __ffs(m) - 1);
-                            qjob[2 * slot] = KEYS ? col | ((uint32_t)row << 8) : (uint32_t)row | (col << 8);
-                            m &= m - 1;
-                            slot++;
-                        }
-                    }
-                    __syncwarp();
-                    run_jobs<kJobSlots>(qjob, min(total, kQCap), stg, Gf, g, lane);
-                    __syncwarp();
-                    // the same candidates in the same order: fold the exact values in
-                    slot = base;
-#pragma unroll 1
-                    for (int c = 0; c < 4 && slot < kQCap; c++) {
-                        uint32_t cm = pick4(pm, c), cx = pick4(px, c);
-                        uint32_t m = cm | cx;
-                        const int bk = (c * 32) / blk;
-                        float emn = pick4(ex_mn, bk), emx = pick4(ex_mx, bk);
-                        while (m && slot < kQCap) {
-                            const uint32_t bit = m & (0u - m);
-                            const float ze = __uint_as_float(qjob[2 * slot + 1]);
-                            if (cm & bit) emn = fminf(emn, ze);
-                            if (cx & bit) emx = fmaxf(emx, ze);
-                            cm &= ~bit;
-                            cx &= ~bit;
-                            m &= m - 1;
-                            slot++;
-                        }
-                        set4(ex_mn, bk, emn);
-                        set4(ex_mx, bk, emx);
-                        set4(pm, c, cm);
-                        set4(px, c, cx);
-                    }
-                    __syncwarp();
-                    pend = (pm[0] | pm[1] | pm[2] | pm[3] | px[0] | px[1] | px[2] | px[3]) != 0;
-                }
-#pragma unroll
-                for (int bk = 0; bk < 4; bk++) {
-                    const int need = (amb >> (2 * bk)) & 3;
-                    if (need) {
-                        m16[bk] = f2h_bits(ex_mn[bk]);
-                        if (need & 1) s16[bk] = scale16(ex_mx[bk], ex_mn[bk], qmaxf);
-                    }
+                if (nj) flush();
+                if (need) {
+                    m16[0] = f2h_bits(ex_mn);
+                    if (need & 1) s16[0] = scale16(ex_mx, ex_mn, qmaxf);
                 }
             }
 
             // ---- 5. code parameters per block
             float rinv[4], c0[4], lim[4];
             int fast = 0;  // bit bk: no value of the block can leave [0, qmax]
-            int live = 0;  // bit bk: finite, non-zero scale (else every code is 0)
 #pragma unroll
             for (int bk = 0; bk < 4; bk++) {
                 rinv[bk] = c0[bk] = 0.0f;
@@ -704,7 +556,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                         lim[bk] = mu < 0.99e-4f ? 2.0f : 0.5f - mu;
                         const float tlo = (mn[bk] - E[bk]) * r + cc, thi = (mx[bk] + E[bk]) * r + cc;
                         if (tlo > -0.49f + mu && thi < qmaxf + 0.49f - mu) fast |= 1 << bk;
-                        live |= 1 << bk;
                     }
                 }
             }
@@ -713,113 +564,107 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
             // rows: the token's codes; keys: the channel's 128-token stream (16 * BITS bytes)
             uint8_t* crow = KEYS ? a.codes + a.cmap.at(ti.l, ti.s, ti.b, ti.h, ti.t0) + (size_t)row * (16 * BITS)
                                  : a.codes + a.cmap.at(ti.l, ti.s, ti.b, ti.h, ti.t0 + row);
-            uint32_t am[4] = {0, 0, 0, 0};  // values within mu of a rounding boundary
+            int nj = 0;  // values within mu of a rounding boundary, to be recomputed exactly and patched
+            // (with masks the row buffer serves the list: 20 jobs and their results)
+            constexpr int kCodeCap = kMasks ? (32 + kJobCap) / 2 : kJobCap;
+            uint32_t* cjobs = kMasks ? reinterpret_cast<uint32_t*>(rowbuf) : jobs;
+            float* cres = kMasks ? rowbuf + kCodeCap : rowbuf;
+            auto patch = [&]() {
+                __syncwarp();
+                tce::run_jobs<kJobSlots>(cjobs, cres, nj, stg, Gf, g, lane);
+                __syncwarp();
+#pragma unroll 1
+                for (int j = 0; j < nj; j++) {
+                    const uint32_t w = cjobs[j];
+                    const float ze = cres[j];
+                    if ((int)((w >> 8) & 31u) == lane)
+                        patch_code<BITS>(crow, (int)(w & 127u) * BITS, quant_code(ze, h2f_bits(s16[0]), h2f_bits(m16[0]), qmax));
+                }
+                __syncwarp();
+                nj = 0;
+            };
+            const float r = rinv[0], cc = c0[0], lm = lim[0];
 #pragma unroll 1
             for (int c = 0; c < 4; c++) {
                 uint32_t v[32];
                 tmem_ld32(tacc + c * 32, v);
                 tmem_wait_ld();
-                const int bk = (c * 32) / blk;
-                const float r = pick4(rinv, bk), cc = pick4(c0, bk), lm = pick4(lim, bk);
-                const bool fst = (fast >> bk) & 1;
-                const bool lv = (live >> bk) & 1;
                 uint32_t words[BITS];
 #pragma unroll
                 for (int w = 0; w < BITS; w++) words[w] = 0;
-                // code k into the packed little-endian stream of this 32-code chunk
-                // y = kMagic + q has the bit pattern 0x4B400000 + q. Widths that straddle words
-                // (3, 6 bits) measure faster with a wrapping sum of y << s per word, less the
-                // constant sum of 0x4B400000 << s; the others mask and OR the codes in.
-                constexpr bool kBiasPack = BITS == 3 || BITS == 6;
-                auto put = [&](int k, uint32_t y) {
-                    const int bit = k * BITS;
-                    if constexpr (kBiasPack) {
-                        words[bit >> 5] += y << (bit & 31);
-                        if ((bit & 31) + BITS > 32) words[(bit >> 5) + 1] += (y & (uint32_t)qmax) >> (32 - (bit & 31));
-                    } else {
-                        const uint32_t q = y & (uint32_t)qmax;
-                        words[bit >> 5] |= q << (bit & 31);
-                        if ((bit & 31) + BITS > 32) words[(bit >> 5) + 1] |= q >> (32 - (bit & 31));
-                    }
-                };
-                uint32_t mk = 0;  // values within mu of a rounding boundary (bit k: column 32c + k)
-                if (fst && lm > 1.0f) {
+                // values within mu of a rounding boundary: whether the lane has one, or a mask of them
+                float worst = 0.0f;
+                uint32_t mask = 0;
+                const float2 r2 = make_float2(r, r), c2 = make_float2(cc, cc), m2 = make_float2(kMagic, kMagic);
+                if ((fast & 1) && lm > 1.0f) {  // no value can need a clamp or lie on the wrong side of a boundary
 #pragma unroll
-                    for (int k = 0; k < 32; k++) put(k, __float_as_uint(fmaf(__uint_as_float(v[k]), r, cc) + kMagic));
+                    for (int k = 0; k < 32; k += 2) {
+                        const float2 t = __ffma2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), r2, c2);
+                        const float2 y = __fadd2_rn(t, m2);
+                        tce::put_code<BITS>(words, k, __float_as_uint(y.x));
+                        tce::put_code<BITS>(words, k + 1, __float_as_uint(y.y));
+                    }
                 } else {
-                    // clamping before the rounding gives the same code as clamping after it
+                    // clamping before the rounding gives the same code as clamping after it (a dead channel: r = c0 = 0, so 0)
 #pragma unroll
-                    for (int k = 31; k >= 0; k--) {
-                        float t = fmaf(__uint_as_float(v[k]), r, cc);
-                        t = fminf(fmaxf(t, 0.0f), qmaxf);
-                        const float y = t + kMagic;
-                        mk = __funnelshift_l(__float_as_uint(__fsub_rn(lm, fabsf(t - (y - kMagic)))), mk, 1);
-                        put(k, lv ? __float_as_uint(y) : 0x4B400000u);  // dead block: q = 0
+                    for (int k = 0; k < 32; k += 2) {
+                        float2 t = __ffma2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), r2, c2);
+                        t = make_float2(fminf(fmaxf(t.x, 0.0f), qmaxf), fminf(fmaxf(t.y, 0.0f), qmaxf));
+                        const float2 y = __fadd2_rn(t, m2);
+                        tce::put_code<BITS>(words, k, __float_as_uint(y.x));
+                        tce::put_code<BITS>(words, k + 1, __float_as_uint(y.y));
+                        const float2 q = __fadd2_rn(y, make_float2(-kMagic, -kMagic));
+                        const float2 e = __ffma2_rn(q, make_float2(-1.0f, -1.0f), t);  // exact
+                        if constexpr (kMasks)
+                            mask |= (fabsf(e.x) > lm ? 1u : 0u) << k | (fabsf(e.y) > lm ? 2u : 0u) << k;
+                        else
+                            worst = max3f(worst, fabsf(e.x), fabsf(e.y));
                     }
                 }
-                if constexpr (kBiasPack) {
 #pragma unroll
-                    for (int w = 0; w < BITS; w++) words[w] -= pack_bias<BITS>(w);
+                for (int w = 0; w < BITS; w++) words[w] -= pack_bias<BITS>(w);
+                uint32_t* dst = reinterpret_cast<uint32_t*>(crow) + c * BITS;
+                if (BITS % 4 == 0) {
+#pragma unroll
+                    for (int w = 0; w < BITS; w += 4)
+                        *reinterpret_cast<uint4*>(dst + w) = make_uint4(words[w], words[w + 1], words[w + 2], words[w + 3]);
+                } else if (BITS % 2 == 0) {
+#pragma unroll
+                    for (int w = 0; w < BITS; w += 2) *reinterpret_cast<uint2*>(dst + w) = make_uint2(words[w], words[w + 1]);
+                } else {
+#pragma unroll
+                    for (int w = 0; w < BITS; w++) dst[w] = words[w];
                 }
-                if (valid) {
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(crow) + c * BITS;
-                    if (BITS % 4 == 0) {
-#pragma unroll
-                        for (int w = 0; w < BITS; w += 4)
-                            *reinterpret_cast<uint4*>(dst + w) = make_uint4(words[w], words[w + 1], words[w + 2], words[w + 3]);
-                    } else if (BITS % 2 == 0) {
-#pragma unroll
-                        for (int w = 0; w < BITS; w += 2) *reinterpret_cast<uint2*>(dst + w) = make_uint2(words[w], words[w + 1]);
-                    } else {
-#pragma unroll
-                        for (int w = 0; w < BITS; w++) dst[w] = words[w];
+                if constexpr (kMasks) {
+                    while (__any_sync(0xffffffffu, mask != 0)) {
+                        const uint32_t word = (uint32_t)(c * 32 + __ffs(mask) - 1) | (uint32_t)row << 8;
+                        const uint32_t left = append(cjobs, kCodeCap, __ballot_sync(0xffffffffu, mask != 0), word, nj);
+                        if (!((left >> lane) & 1u)) mask &= mask - 1;
+                        if (left) patch();  // the list is full
+                    }
+                } else {
+                    uint32_t todo = __ballot_sync(0xffffffffu, worst > lm);
+                    uint32_t left = 0xffffffffu;
+                    while (todo) {
+                        tmem_ld32(tacc + c * 32, v);
+                        tmem_wait_ld();
+                        do {
+                            const int src = __ffs(todo) - 1;
+                            const float sr = __shfl_sync(0xffffffffu, r, src), sc = __shfl_sync(0xffffffffu, cc, src);
+                            const float sl = __shfl_sync(0xffffffffu, lm, src);
+                            const float z = spread(v, src);
+                            const float t = fminf(fmaxf(fmaf(z, sr, sc), 0.0f), qmaxf);
+                            left = append(cjobs, kCodeCap, __ballot_sync(0xffffffffu, fabsf(t - ((t + kMagic) - kMagic)) > sl) & left,
+                                          (uint32_t)(c * 32 + lane) | (uint32_t)(q4 * 32 + src) << 8, nj);
+                            if (left) break;  // the list is full
+                            todo &= todo - 1;
+                            left = 0xffffffffu;
+                        } while (todo);
+                        if (todo) patch();
                     }
                 }
-                if (valid && lv) set4(am, c, mk);
             }
-            bool pend = (am[0] | am[1] | am[2] | am[3]) != 0;
-            while (__any_sync(0xffffffffu, pend)) {
-                const int cnt = __popc(am[0]) + __popc(am[1]) + __popc(am[2]) + __popc(am[3]);
-                int inc = cnt;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, inc, off);
-                    if (lane >= off) inc += t;
-                }
-                const int base = inc - cnt;
-                const int total = __shfl_sync(0xffffffffu, inc, 31);
-                int slot = base;
-#pragma unroll 1
-                for (int c = 0; c < 4 && slot < kQCap; c++) {
-                    uint32_t m = pick4(am, c);
-                    while (m && slot < kQCap) {
-                        const uint32_t col = (uint32_t)(c * 32 + __ffs(m) - 1);
-                        qjob[2 * slot] = KEYS ? col | ((uint32_t)row << 8) : (uint32_t)row | (col << 8);
-                        m &= m - 1;
-                        slot++;
-                    }
-                }
-                __syncwarp();
-                run_jobs<kJobSlots>(qjob, min(total, kQCap), stg, Gf, g, lane);
-                __syncwarp();
-                slot = base;
-#pragma unroll 1
-                for (int c = 0; c < 4 && slot < kQCap; c++) {
-                    uint32_t m = pick4(am, c);
-                    while (m && slot < kQCap) {
-                        const int col = c * 32 + __ffs(m) - 1;
-                        const float ze = __uint_as_float(qjob[2 * slot + 1]);
-                        const int bk = col / blk;
-                        const uint32_t q = quant_code(ze, h2f_bits(pick4(s16, bk)), h2f_bits(pick4(m16, bk)), qmax);
-                        patch_code<BITS>(crow, col * BITS, q);
-                        m &= m - 1;
-                        slot++;
-                    }
-                    set4(am, c, m);
-                }
-                __syncwarp();
-                pend = (am[0] | am[1] | am[2] | am[3]) != 0;
-            }
+            if (nj) patch();
 
             // ---- 7. scales; release the stage and the accumulator buffer
             if (valid) {
