@@ -286,16 +286,17 @@ __global__ void __launch_bounds__(kAThreads) attn_chunk_kernel(AttnArgs a) {
     }
 }
 
-constexpr int kCThreads = 512;   // merge: 128 channels x 4 slices of the parts and of the rotation
 constexpr int kCParts = 256;     // parts whose weights are held at a time
 
 // Merges the parts of one (l, b, h) and applies G_V^T (per gauge group): out fp32. It waits for
 // memory, not arithmetic: the parts' maxima, sums and weights are taken one per thread, so that the
 // loop over the parts only loads their value sums, 4 n_rep of a thread in flight; a slice's gauge
-// values are loaded first. 8 units of 57 parts: 17 -> 6 us.
-template <int NREP>
-__global__ void __launch_bounds__(kCThreads) attn_combine_kernel(AttnArgs a) {
-    __shared__ float red[4][NREP][kAD], zs[NREP][kAD], Mw[kCThreads / 32][NREP], Lw[kCThreads / 32][NREP];
+// values are loaded first. 8 units of 57 parts: 17 -> 6 us. Threads: 128 channels x SL slices of the parts and
+// of the rotation (launch_combine).
+template <int NREP, int SL>
+__global__ void __launch_bounds__(SL * kAD) attn_combine_kernel(AttnArgs a) {
+    constexpr int kCThreads = SL * kAD;
+    __shared__ float red[SL][NREP][kAD], zs[NREP][kAD], Mw[kCThreads / 32][NREP], Lw[kCThreads / 32][NREP];
     __shared__ float wgt[kCParts][NREP];
     const int unit = blockIdx.x, tid = threadIdx.x, c = tid & (kAD - 1), sl = tid >> 7, lane = tid & 31;
     const int l = unit / (a.B * a.H), h = unit % a.H;
@@ -303,11 +304,15 @@ __global__ void __launch_bounds__(kCThreads) attn_combine_kernel(AttnArgs a) {
     constexpr int kStride = NREP * (kAD + 2);
     const float* part = a.part + (int64_t)unit * a.n_parts * kStride;
     const int n_parts = (int)(((unit + 1) * a.unit_steps - 1) / a.cta_steps - unit * a.unit_steps / a.cta_steps) + 1;
-    const int per = g / 4;  // g >= 8: gauge rows of this slice
+    const int per = g / SL;  // g >= 8: gauge rows of this slice
     const float* Gv = a.G + ((int64_t)(l * 2 + 1) * a.H + h) * (int64_t)kAD * g + (int64_t)grp * g * g + (int64_t)sl * per * g + i;
     float gv[32];
 #pragma unroll
     for (int j = 0; j < 32; j++) gv[j] = j < per ? __ldg(Gv + (int64_t)j * g) : 0.0f;
+    auto slices = [&](int r, int k) -> float {
+        if constexpr (SL == 1) return red[0][r][k];
+        else return (red[0][r][k] + red[1][r][k]) + (red[2][r][k] + red[3][r][k]);
+    };
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the parts
     float m = -INFINITY;  // thread: query tid mod NREP
     for (int e = tid; e < n_parts * NREP; e += kCThreads) m = fmaxf(m, part[(int64_t)e * (kAD + 2)]);
@@ -330,7 +335,7 @@ __global__ void __launch_bounds__(kCThreads) attn_combine_kernel(AttnArgs a) {
         }
         __syncthreads();
 #pragma unroll 4
-        for (int j = sl; j < n; j += 4)
+        for (int j = sl; j < n; j += SL)
 #pragma unroll
             for (int r = 0; r < NREP; r++) o[r] = fmaf(p0[(int64_t)j * kStride + r * (kAD + 2) + 2 + c], wgt[j][r], o[r]);
         __syncthreads();
@@ -346,7 +351,7 @@ __global__ void __launch_bounds__(kCThreads) attn_combine_kernel(AttnArgs a) {
         float s = 0.0f;
 #pragma unroll
         for (int w = 0; w < kCThreads / 32; w++) s += Lw[w][r];
-        zs[r][k] = ((red[0][r][k] + red[1][r][k]) + (red[2][r][k] + red[3][r][k])) / s;
+        zs[r][k] = slices(r, k) / s;
     }
     __syncthreads();
 #pragma unroll
@@ -356,12 +361,14 @@ __global__ void __launch_bounds__(kCThreads) attn_combine_kernel(AttnArgs a) {
 #pragma unroll
         for (int j = 0; j < 32; j++)
             if (j < per) s = fmaf(gv[j], z[j], s);
+        if constexpr (SL == 1)
+            for (int j = 32; j < per; j++) s = fmaf(__ldg(Gv + (int64_t)j * g), z[j], s);
         red[sl][r][c] = s;
     }
     __syncthreads();
     for (int e = tid; e < NREP * kAD; e += kCThreads) {
         const int r = e / kAD, k = e % kAD;
-        a.out[((int64_t)unit * NREP + r) * kAD + k] = (red[0][r][k] + red[1][r][k]) + (red[2][r][k] + red[3][r][k]);
+        a.out[((int64_t)unit * NREP + r) * kAD + k] = slices(r, k);
     }
 }
 
@@ -1044,6 +1051,16 @@ cudaError_t launch_chunks_bits(const AttnArgs& a, cudaStream_t st) {
     }
 }
 
+// Few units: four slices of the parts and of the rotation per unit, for latency. More than two wide
+// CTAs per SM would come in waves, so those get one slice each (768 units of 12 parts, 3 bits, whole call:
+// 194.7 us with four slices, 182.5 with one; 512 units of 16,384 tokens: 280.7 and 281.4).
+template <int NREP>
+cudaError_t launch_combine(const AttnArgs& a, int sms, cudaStream_t st) {
+    const int64_t units = (int64_t)a.L * a.B * a.H;
+    if (units > 2 * (int64_t)sms) return launch_dependent(attn_combine_kernel<NREP, 1>, (unsigned)units, kAD, 0, a, st);
+    return launch_dependent(attn_combine_kernel<NREP, 4>, (unsigned)units, 4 * kAD, 0, a, st);
+}
+
 }  // namespace
 
 size_t attn_workspace_bytes(int64_t units, int n_rep, int d, int64_t T) {
@@ -1074,12 +1091,11 @@ cudaError_t launch_attention(const AttnArgs& args, cudaStream_t st) {
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    const unsigned units = (unsigned)(a.L * a.B * a.H);
     switch (a.n_rep) {
-        case 1: return launch_dependent(attn_combine_kernel<1>, units, kCThreads, 0, a, st);
-        case 2: return launch_dependent(attn_combine_kernel<2>, units, kCThreads, 0, a, st);
-        case 4: return launch_dependent(attn_combine_kernel<4>, units, kCThreads, 0, a, st);
-        case 8: return launch_dependent(attn_combine_kernel<8>, units, kCThreads, 0, a, st);
+        case 1: return launch_combine<1>(a, sms, st);
+        case 2: return launch_combine<2>(a, sms, st);
+        case 4: return launch_combine<4>(a, sms, st);
+        case 8: return launch_combine<8>(a, sms, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -63,3 +63,10 @@ def test_value_scales(first, later, n_rep):
         return s.reshape(-1).view(np.uint16)
 
     _check(w, n_rep, w.T, scales=scales)
+
+
+@pytest.mark.parametrize("bits,n_rep", [(3, 1), (4, 2), (6, 4), (4, 8)])
+@pytest.mark.parametrize("B,group", [(76, 128), (77, 128), (77, 8)])
+def test_merge_widths(bits, n_rep, B, group):
+    """304 units of several parts (two per SM: four slices merge a unit) and 308 (one slice)."""
+    _check(_wl(T=290, bits=bits, group=group, L=1, B=B, H=4), n_rep, 290)
