@@ -251,8 +251,10 @@ __global__ void __launch_bounds__(kThreads, kCtas) hadamard_encode_kernel(const 
             mx[sb] = hi;
         }
         // an Inf or NaN input makes all (at least 8) values of its group Inf or NaN, and this sum of one
-        // value of each eight too; huge finite values can overflow as well: look at the input
-        if (!isfinite((v[0].x + v[8].x) + (v[0].y + v[8].y))) {
+        // value of each eight too; huge finite values can overflow as well: look at the input. The lane's
+        // codes then come from exact_code, which knows NaN (min and max pass over one)
+        bool plain = isfinite((v[0].x + v[8].x) + (v[0].y + v[8].y));
+        if (!plain) {
             for (int q = 0; q < 4; q++) {
                 const uint4 x = *reinterpret_cast<const uint4*>(src + 16 * q);
                 const uint32_t w[4] = {x.x, x.y, x.z, x.w};
@@ -266,7 +268,6 @@ __global__ void __launch_bounds__(kThreads, kCtas) hadamard_encode_kernel(const 
         // scales, and whether every code is a plain rounding (no clamp, no quotient near a half-integer)
         uint32_t sz[NSUB];
         float m[NSUB], r[NSUB];
-        bool plain = true;
 #pragma unroll
         for (int sb = 0; sb < NSUB; sb++) {
             sz[sb] = scale_bits<BITS>(__fsub_rn(mx[sb], mn[sb])) | (f2h_bits(mn[sb]) << 16);
