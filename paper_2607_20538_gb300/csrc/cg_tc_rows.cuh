@@ -599,7 +599,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
             for (int bk = 0; bk < NBK; bk++) {
                 rinv[bk] = c0[bk] = 0.0f;
                 lim[bk] = 0.5f;
-                fast[bk] = true;  // a dead block (zero or overflowing scale) codes to 0 with r = c0 = 0
+                // a dead block (zero or overflowing scale) codes to 0 with r = c0 = 0, unless its z~ may not be
+                // finite: NaN takes the checked loop, whose clamp makes it 0
+                fast[bk] = Ec[bk] < INFINITY;
                 if (valid && (h_is_inf(s16[bk]) || h_is_inf(m16[bk]))) flag |= CG_FLAG_FP16_OVERFLOW;
                 const float sc = h2f_bits(s16[bk]), mz = h2f_bits(m16[bk]);
                 if constexpr (TILE) {

@@ -48,6 +48,24 @@ def _wl(backend, T, bits, group, block):
     return synth.Workload("nonfinite", L=1, B=2, H=2, T=T, d=128, group=group, backend=backend, bits=bits, block=block, residual=0)
 
 
+@pytest.mark.parametrize("value", VALUES[:3])
+@pytest.mark.parametrize("bits,group,block", [(8, 64, 32), (8, 128, 128), (8, 32, 32), (4, 128, 64), (3, 32, 32)])
+def test_row_codes_of_blocks_without_a_scale(value, bits, group, block):
+    """A row's block that holds no finite range codes to 0; its neighbours keep their codes."""
+    w = _wl(0, 200, bits, group, block)
+    places = [(0, 3, 5), (1, 199, 127), (2, 17, 40), (3, 100, 0), (5, 64, 66)]
+    codes, scales, ref = _encode(w, value, places)
+    q = lambda b: np.unpackbits(b.reshape(-1, w.T, 128 * bits // 8), axis=-1, bitorder="little").reshape(-1, w.T, 128, bits)
+    got, want = q(codes), q(ref["codes"])
+    for u, t, c in places:  # blocks that share channels with the value's gauge group
+        r = np.arange(128) // group == c // group
+        own = np.repeat(r.reshape(-1, block).any(1), block)
+        assert not got[u, t, own].any()
+        got[u, t], want[u, t] = 0, 0
+    flagged = ref["flags"].reshape(got.shape[:3]).astype(bool)
+    assert flagged[(got != want).any(-1)].all()
+
+
 @pytest.mark.parametrize("value", VALUES)
 @pytest.mark.parametrize("bits,group,block", [(4, 8, 128), (3, 16, 32), (2, 32, 64), (3, 8, 32), (8, 16, 128)])
 def test_hadamard(value, bits, group, block):
