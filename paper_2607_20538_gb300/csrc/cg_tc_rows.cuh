@@ -488,7 +488,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                 float er = Ec[bk];  // the bound of the range: the row's, or the largest of the tile's rows
                 if constexpr (TILE) {
                     // a range covers the 16 rows of a tile, which are 16 lanes of this warp; rows
-                    // that do not exist take no part
+                    // that do not exist take no part. A row with an Inf or NaN (or squares beyond fp32) has
+                    // no bound, and a NaN z~ where the exact z may be anything: the whole tile is undecided
+                    if (!(er < INFINITY)) er = INFINITY;
                     if (!valid) {
                         mn[bk] = INFINITY;
                         mx[bk] = -INFINITY;
@@ -552,8 +554,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     const int need = (amb >> (2 * bk)) & 3;
                     const float e2 = 2.0f * pickn(E, bk);
                     float tl = __fadd_rn(pickn(mn, bk), e2), th = __fsub_rn(pickn(mx, bk), e2);
-                    const bool nl = need != 0 && pickn(cmn, c) <= tl;
-                    const bool nh = (need & 1) && pickn(cmx, c) >= th;
+                    // (tiles: a NaN z~ is a candidate, for which only the exact value can tell)
+                    const bool nl = need != 0 && (TILE ? !(pickn(cmn, c) > tl) : pickn(cmn, c) <= tl);
+                    const bool nh = (need & 1) && (TILE ? !(pickn(cmx, c) < th) : pickn(cmx, c) >= th);
                     uint32_t todo = __ballot_sync(0xffffffffu, nl || nh);
                     if (todo == 0) continue;
                     if (!nl) tl = -INFINITY;
@@ -567,8 +570,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                             const int src = __ffs(todo) - 1;
                             const float stl = __shfl_sync(0xffffffffu, tl, src), sth = __shfl_sync(0xffffffffu, th, src);
                             const float z = spread(v, src);
+                            const bool low = TILE ? !(z > stl) : z <= stl, high = TILE ? !(z < sth) : z >= sth;
                             const uint32_t job = (uint32_t)(q4 * 32 + src) | (uint32_t)(c * 32 + lane) << 8 |
-                                                 (z <= stl ? 0x10000u : 0u) | (z >= sth ? 0x20000u : 0u);
+                                                 (low ? 0x10000u : 0u) | (high ? 0x20000u : 0u);
                             left = append(__ballot_sync(0xffffffffu, (job & 0x30000u) != 0u) & left, job, nj);
                             if (left) break;  // the list is full
                             todo &= todo - 1;
@@ -584,6 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     if constexpr (TILE) {
                         ex_mn[bk] = half_warp_min(ex_mn[bk]);
                         ex_mx[bk] = half_warp_max(ex_mx[bk]);
+                        if ((need & 1) && ex_mn[bk] > ex_mx[bk]) ex_mn[bk] = ex_mx[bk] = NAN;  // no value but NaN
                     }
                     if (need) {
                         m16[bk] = f2h_bits(ex_mn[bk]);
@@ -605,6 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                 if (valid && (h_is_inf(s16[bk]) || h_is_inf(m16[bk]))) flag |= CG_FLAG_FP16_OVERFLOW;
                 const float sc = h2f_bits(s16[bk]), mz = h2f_bits(m16[bk]);
                 if constexpr (TILE) {
+                    if (!fast[bk]) lim[bk] = -1.0f;  // no bound: every code of the row is recomputed
                     // the rule's code of a finite value over a zero of -inf: fl((z + inf) / s) clamps to qmax
                     if (m16[bk] == 0xfc00u && sc != 0.0f && !h_is_inf(s16[bk])) c0[bk] = qmaxf;
                 }
@@ -619,7 +625,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     const float mu = Ec[bk] * r * 1.0001f + (zr + 2.0f * fabsf(cc) + 3.0f * (qmaxf + 1.0f)) * 6.6e-8f;
                     // mu < 1e-4: a code from z~ can only differ where the tolerance allows it (tiles:
                     // every code is the exact rule's)
-                    lim[bk] = !TILE && mu < 0.99e-4f ? 2.0f : 0.5f - mu;
+                    // (fmaxf: without a bound every code)
+                    lim[bk] = TILE ? fmaxf(0.5f - mu, -1.0f) : (mu < 0.99e-4f ? 2.0f : 0.5f - mu);
                     const float tlo = (mn[bk] - E[bk]) * r + cc, thi = (mx[bk] + E[bk]) * r + cc;
                     fast[bk] = tlo > -0.49f + mu && thi < qmaxf + 0.49f - mu && (kTrack || lim[bk] > 1.0f);
                 }

@@ -48,6 +48,16 @@ def _wl(backend, T, bits, group, block):
     return synth.Workload("nonfinite", L=1, B=2, H=2, T=T, d=128, group=group, backend=backend, bits=bits, block=block, residual=0)
 
 
+@pytest.mark.parametrize("value", VALUES)
+@pytest.mark.parametrize("bits,group,block", [(4, 128, 128), (4, 8, 128), (3, 16, 32), (2, 32, 64), (8, 64, 32)])
+def test_tiles(value, bits, group, block):
+    w = _wl(3, 200, bits, group, block)
+    places = [(0, 3, 5), (1, 199, 127), (2, 17, 40), (3, 100, 1)] + [(5, t, 66) for t in range(33, 48)] + [(6, 64 + t, 9 * t) for t in range(1, 14)]
+    codes, scales, ref = _encode(w, value, places)
+    np.testing.assert_array_equal(scales, ref["scales"].view(np.float16))
+    np.testing.assert_array_equal(codes, ref["codes"])
+
+
 @pytest.mark.parametrize("value", VALUES[:3])
 @pytest.mark.parametrize("bits,group,block", [(8, 64, 32), (8, 128, 128), (8, 32, 32), (4, 128, 64), (3, 32, 32)])
 def test_row_codes_of_blocks_without_a_scale(value, bits, group, block):
