@@ -409,6 +409,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                             if (bf16_nonfinite(wv[k] & 0xffffu) || bf16_nonfinite(wv[k] >> 16))
                                 flag |= CG_FLAG_NONFINITE_INPUT;
                     }
+                    // no bound for the tile's channels: the MMA's zero blocks times Inf or NaN spoil the
+                    // token's z~ in every group, so all groups are undecided and every code is recomputed
+                    for (int rr = 0; rr < 4; rr++) gs[rr] = INFINITY;
                 }
 #pragma unroll
                 for (int rr = 0; rr < 4; rr++)
@@ -431,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
 #pragma unroll
                 for (int rr = 0; rr < 4; rr++)
                     gm[rr] = fmaxf(fmaxf(xb[rr], xb[4 + rr]), fmaxf(xb[8 + rr], xb[12 + rr]));
-                bs[0] = pick4(gm, row / g);  // fmaxf keeps a NaN out; non-finite input is flagged above
+                bs[0] = pick4(gm, row / g);
             }
             // ---- 2. approximate range of the channel from the accumulator, per 32-token chunk and whole
             static_assert(NBK == 1, "one block per channel");
@@ -502,8 +505,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                 const float e2 = 2.0f * E[0], tl0 = __fadd_rn(mn[0], e2), th0 = __fsub_rn(mx[0], e2);
 #pragma unroll 1
                 for (int c = 0; c < 4; c++) {
-                    const bool nl = need != 0 && pick4(cmn, c) <= tl0;
-                    const bool nh = (need & 1) && pick4(cmx, c) >= th0;
+                    const bool nl = need != 0 && !(pick4(cmn, c) > tl0);  // a NaN z~ is a candidate
+                    const bool nh = (need & 1) && !(pick4(cmx, c) < th0);
                     uint32_t todo = __ballot_sync(0xffffffffu, nl || nh);
                     if (todo == 0) continue;
                     const float tl = nl ? tl0 : -INFINITY, th = nh ? th0 : INFINITY;
@@ -517,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                             const float stl = __shfl_sync(0xffffffffu, tl, src), sth = __shfl_sync(0xffffffffu, th, src);
                             const float z = spread(v, src);
                             const uint32_t job = (uint32_t)(c * 32 + lane) | (uint32_t)(q4 * 32 + src) << 8 |
-                                                 (z <= stl ? 0x10000u : 0u) | (z >= sth ? 0x20000u : 0u);
+                                                 (z > stl ? 0u : 0x10000u) | (z < sth ? 0u : 0x20000u);
                             left = append(jobs, kJobCap, __ballot_sync(0xffffffffu, (job & 0x30000u) != 0u) & left, job, nj);
                             if (left) break;  // the list is full
                             todo &= todo - 1;
@@ -553,7 +556,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                         const float zr = fmaxf(fabsf(mn[bk]), fabsf(mx[bk])) * r;
                         const float mu = E[bk] * r * 1.0001f + (zr + 2.0f * fabsf(cc) + 3.0f * (qmaxf + 1.0f)) * 6.6e-8f;
                         // mu < 1e-4: a code from z~ can only differ where the tolerance allows it
-                        lim[bk] = mu < 0.99e-4f ? 2.0f : 0.5f - mu;
+                        // (fmaxf: without a bound every code is recomputed)
+                        lim[bk] = mu < 0.99e-4f ? 2.0f : fmaxf(0.5f - mu, -1.0f);
                         const float tlo = (mn[bk] - E[bk]) * r + cc, thi = (mx[bk] + E[bk]) * r + cc;
                         if (tlo > -0.49f + mu && thi < qmaxf + 0.49f - mu) fast |= 1 << bk;
                     }

@@ -12,6 +12,8 @@ import pytest
 import oracle
 from paper_2607_20538_gb300 import synth
 
+from cgcheck import compare_codes
+
 torch = pytest.importorskip("torch")
 cg = pytest.importorskip("paper_2607_20538_gb300")
 
@@ -74,6 +76,16 @@ def test_row_codes_of_blocks_without_a_scale(value, bits, group, block):
         got[u, t], want[u, t] = 0, 0
     flagged = ref["flags"].reshape(got.shape[:3]).astype(bool)
     assert flagged[(got != want).any(-1)].all()
+
+
+@pytest.mark.parametrize("value", VALUES)
+@pytest.mark.parametrize("bits,group", [(2, 32), (4, 128), (3, 64), (8, 64), (6, 32)])
+def test_keys(value, bits, group):
+    w = _wl(1, 256, bits, group, 128)
+    places = [(0, 3, 5), (1, 127, 127), (2, 130, 40), (2, 255, 0), (3, 200, 64)]  # units 0..3 hold the keys
+    codes, scales, ref = _encode(w, value, places)
+    np.testing.assert_array_equal(scales, ref["scales"].view(np.float16))
+    compare_codes(w, codes, ref["codes"], ref["flags"])
 
 
 @pytest.mark.parametrize("value", VALUES)
