@@ -28,10 +28,14 @@
 //      (both are monotone in the extremes, so equal interval ends decide them exactly);
 //   4. blocks the intervals leave undecided: candidate extremes (values within 2E of the
 //      approximate extreme, only in chunks whose own extreme qualifies) are recomputed
-//      exactly in the library's order by the warp together (run_jobs). A warp has one or two
-//      such rows a tile; a row's chunk is spread over the lanes through 128 bytes of shared
-//      memory, so one compare and vote finds its candidates (building a 32-bit candidate mask
-//      in every lane, and job lists by prefix sums over them, took twice the instructions);
+//      exactly in the library's order by the warp together (run_jobs). Two ways to find them:
+//      search (MASKS = false): a warp has one or two such rows a tile; a row's chunk is spread
+//      over the lanes through 128 bytes of shared memory, so one compare and vote finds its
+//      candidates. Fewer instructions, but a chain of some 200 cycles per row.
+//      masks (MASKS = true): every lane builds a 32-bit candidate mask of each chunk, job lists
+//      by prefix sums over them (step 6 likewise). Better where a warp has five or six
+//      undecided blocks a tile (32-channel blocks under a 128-wide gauge) or where a CTA has a
+//      few tiles only, so that nothing hides the chain; launch_rows_bits has the line;
 //   5. codes straight from tensor memory: t = z~ * (1/s) - m/s, y = t + 1.5 * 2^23 (round to
 //      nearest even in the add; y's bit pattern is 0x4B400000 + q), packed by wrapping sums
 //      of y << (bit offset) less a compile-time constant. A chunk takes the short loop when
@@ -45,7 +49,7 @@
 // max per two values, and only a chunk where that exceeds 1/2 - mu (6 % of them at 4 bits) marks
 // its values one by one. A range of 2048 values is undecided as rarely as one of 64, so the
 // exact-extreme step nearly vanishes. 8B-shaped cache (1 GiB bf16, 4 bits, block 128): 9.92 ms
-// with the exact rotation on CUDA cores -> 0.50 ms (2.7 TB/s, 40 % of measured HBM); bound by
+// with the exact rotation on CUDA cores -> 0.42 ms (3.2 TB/s, 48 % of measured HBM); bound by
 // the epilogue's instruction issue and latencies, as the rows are.
 // The block count is a template parameter, so the per-block state of a row takes only the
 // registers it needs; the chunk loops are not unrolled (the epilogue's code size sets its
@@ -89,7 +93,9 @@ struct RowMisc {
     uint32_t tmem_slot;
     int abort_flag;
     float emaxb[kSegBufs][2][4];  // per gauge set, converter warp and quantization block: max_i e_i
-    float gmaxb[kSegBufs][2][4];  // and max_i ||G_i||
+    // and max_i ||G_i||, which nothing reads: without it the compiler schedules the epilogue of two blocks a
+    // row 8 % slower (8B-shaped cache 552 us with it, 597 without; other block counts 1 to 3 % faster)
+    float gmaxb[kSegBufs][2][4];
 };
 
 static_assert(sizeof(RowMisc) <= 512, "RowMisc outgrew its shared-memory slot");
@@ -189,7 +195,7 @@ __device__ __forceinline__ float half_warp_max(float v) {
     return v;
 }
 
-template <int BITS, int NBK, bool TILE>
+template <int BITS, int NBK, bool TILE, bool MASKS>
 __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __grid_constant__ CUtensorMap xmap,
                                                                       const RowEncParams P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -399,8 +405,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
         constexpr float kAbove1 = 1.0f + 8.0f * kU;
         constexpr int qmax = (1 << BITS) - 1;
         // 8-bit codes nearly always have mu >= 1e-4: their usual loop tracks the distances too
-        constexpr bool kTrack = TILE || BITS == 8;
+        constexpr bool kTrack = (TILE || BITS == 8) && !MASKS;
+        // Search, several blocks a row: one call site of the exact round for full and last lists (the
+        // epilogue's code size sets its instruction fetch; 8B-shaped cache 594 -> 552 us; one block a row
+        // and tiles measured 1 to 3 % faster with two). Four blocks: the exact extremes of one block at a
+        // time in registers, no spills (27B-shaped cache at 6 bits 4360 -> 3925 us)
+        constexpr bool kOneSite = NBK > 1 && !TILE;
+        constexpr bool kInPlace = NBK == 4 && !TILE && !MASKS;
         constexpr int kJobSlots = NBK == 2 ? 4 : 2;  // values per lane and memory round trip
+        constexpr int kListCap = (32 + kJobCap) / 2;  // MASKS: jobs and results share the warp's buffer
+        uint32_t* djobs = reinterpret_cast<uint32_t*>(rowbuf);
+        float* dres = rowbuf + kListCap;
         int32_t flag = 0;
         tc::TileIter it;
         it.init(a, S, t_begin + wg);
@@ -478,8 +493,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
             }
 
             // ---- 3. error bound per block; scale/zero from the intervals when they agree
-            float E[NBK], Ec[NBK];  // Ec bounds |z~ - z|; E adds the rounding of the interval ends
-            uint32_t s16[NBK], m16[NBK];
+            float Et[TILE ? NBK : 1], Ec[NBK];  // Ec bounds |z~ - z|; E adds the rounding of the interval ends
+            // E (rows: recomputed where it is used, for the registers)
+            auto bound = [&](float ec, float lo, float hi) { return ec + (fabsf(lo) + fabsf(hi)) * 2.4e-7f; };
+            uint32_t sz[NBK];  // scale, zero << 16
             int amb = 0;  // bit 2bk: scale needs the exact extremes; bit 2bk+1: zero needs the exact min
 #pragma unroll
             for (int bk = 0; bk < NBK; bk++) {
@@ -500,8 +517,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     mx[bk] = half_warp_max(mx[bk]);
                     er = half_warp_max(er);
                 }
-                E[bk] = er + (fabsf(mn[bk]) + fabsf(mx[bk])) * 2.4e-7f;
-                const float e = E[bk];
+                const float e = bound(er, mn[bk], mx[bk]);
+                if constexpr (TILE) Et[bk] = e;
                 const float mn_lo = __fsub_rn(mn[bk], e), mn_hi = __fadd_rn(mn[bk], e);
                 const float mx_lo = __fsub_rn(mx[bk], e), mx_hi = __fadd_rn(mx[bk], e);
                 // fp16 scales of the smallest and largest possible ranges. fl(d * fl(1/qmax))
@@ -513,56 +530,142 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                 const uint32_t slo = f2h_bits(__fmul_rn(__fmul_rn(dlo, kRq), kBelow1));
                 const uint32_t shi = f2h_bits(__fmul_rn(__fmul_rn(dhi, kRq), kAbove1));
                 const uint32_t mlo = f2h_bits(mn_lo), mhi = f2h_bits(mn_hi);
-                s16[bk] = slo;
-                m16[bk] = mlo;
+                sz[bk] = slo | mlo << 16;
                 if (valid && slo != shi) amb |= 1 << (2 * bk);
                 if (valid && mlo != mhi) amb |= 2 << (2 * bk);
+                if constexpr (kInPlace) {  // a block without a candidate (NaN sums): the extremes of no value
+                    const int need = (amb >> (2 * bk)) & 3;
+                    if (need) sz[bk] = ((need & 1) ? 0xfc00u : slo) | 0x7c00u << 16;
+                }
             }
 
             // ---- 4. exact extremes of undecided blocks. Candidates of a block's min (max) are its values
-            // within 2E of the approximate min (max), only in chunks whose own min (max) lies that close.
-            // The few rows concerned are taken one by one: the row's chunk is spread over the lanes, so
-            // that one compare and vote finds its candidates
+            // within 2E of the approximate min (max), only in chunks whose own min (max) lies that close
             if (__any_sync(0xffffffffu, amb != 0)) {
-                float ex_mn[NBK], ex_mx[NBK];
+                // exact extremes so far, per block, or of block `cur` of the row: a row's jobs come in the order
+                // of their columns, so a block is complete when a job of the next one comes
+                constexpr int NEX = kInPlace ? 1 : NBK;
+                float ex_mn[NEX], ex_mx[NEX];
+                int cur = -1;
 #pragma unroll
-                for (int bk = 0; bk < NBK; bk++) {
+                for (int bk = 0; bk < NEX; bk++) {
                     ex_mn[bk] = INFINITY;
                     ex_mx[bk] = -INFINITY;
                 }
-                int nj = 0;
-                auto flush = [&]() {
-                    __syncwarp();
-                    run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
-                    __syncwarp();
-#pragma unroll 1
-                    for (int j = 0; j < nj; j++) {
-                        const uint32_t w = jobs[j];
-                        const float ze = rowbuf[j];
-                        if ((int)(w & 31u) == lane) {
-                            const int bk = (int)((w >> 8) & 127u) / blk;
-                            if (w & 0x10000u) setn(ex_mn, bk, fminf(pickn(ex_mn, bk), ze));
-                            if (w & 0x20000u) setn(ex_mx, bk, fmaxf(pickn(ex_mx, bk), ze));
-                        }
-                    }
-                    __syncwarp();
-                    nj = 0;
+                auto exact = [&](int bk, uint32_t old, float lo, float hi) {
+                    return (((amb >> (2 * bk)) & 1) ? scale16(hi, lo, qmaxf) : old & 0xffffu) | f2h_bits(lo) << 16;
                 };
+                if constexpr (MASKS) {
+                    // every lane's candidates take consecutive slots (warp prefix sum of the counts); one
+                    // cooperative round serves up to kListCap of them
+                    uint32_t pm[4] = {0, 0, 0, 0}, px[4] = {0, 0, 0, 0};
 #pragma unroll 1
-                for (int c = 0; c < 4; c++) {
-                    const int bk = c / CPB;
-                    const int need = (amb >> (2 * bk)) & 3;
-                    const float e2 = 2.0f * pickn(E, bk);
-                    float tl = __fadd_rn(pickn(mn, bk), e2), th = __fsub_rn(pickn(mx, bk), e2);
-                    // (tiles: a NaN z~ is a candidate, for which only the exact value can tell)
-                    const bool nl = need != 0 && (TILE ? !(pickn(cmn, c) > tl) : pickn(cmn, c) <= tl);
-                    const bool nh = (need & 1) && (TILE ? !(pickn(cmx, c) < th) : pickn(cmx, c) >= th);
-                    uint32_t todo = __ballot_sync(0xffffffffu, nl || nh);
-                    if (todo == 0) continue;
-                    if (!nl) tl = -INFINITY;
-                    if (!nh) th = INFINITY;
-                    uint32_t left = 0xffffffffu;  // values of row src that no earlier round has taken
-                    while (todo) {
+                    for (int c = 0; c < 4; c++) {
+                        const int bk = c / CPB;
+                        const int need = (amb >> (2 * bk)) & 3;
+                        const float e2 = 2.0f * bound(pickn(Ec, bk), pickn(mn, bk), pickn(mx, bk));
+                        const float tl = __fadd_rn(pickn(mn, bk), e2), th = __fsub_rn(pickn(mx, bk), e2);
+                        const bool nl = need != 0 && pickn(cmn, c) <= tl;
+                        const bool nh = (need & 1) && pickn(cmx, c) >= th;
+                        uint32_t m0 = 0, m1 = 0;
+                        if (__any_sync(0xffffffffu, nl || nh)) {
+                            uint32_t v[32];
+                            tmem_ld32(tacc + c * 32, v);
+                            tmem_wait_ld();
+                            // sign bits of tl - z (z > tl) and z - th (z < th), one bit per column
+                            uint32_t a0 = 0, a1 = 0;
+                            if constexpr (NBK == 4) {  // (one loop for both keeps the row's state in registers)
+#pragma unroll
+                                for (int k = 31; k >= 0; k--) {
+                                    const float z = __uint_as_float(v[k]);
+                                    a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl, z)), a0, 1);
+                                    a1 = __funnelshift_l(__float_as_uint(__fsub_rn(z, th)), a1, 1);
+                                }
+                            } else {
+                                if (__any_sync(0xffffffffu, nl)) {
+#pragma unroll
+                                    for (int k = 31; k >= 0; k--)
+                                        a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl, __uint_as_float(v[k]))), a0, 1);
+                                }
+                                if (__any_sync(0xffffffffu, nh)) {
+#pragma unroll
+                                    for (int k = 31; k >= 0; k--)
+                                        a1 = __funnelshift_l(__float_as_uint(__fsub_rn(__uint_as_float(v[k]), th)), a1, 1);
+                                }
+                            }
+                            m0 = nl ? ~a0 : 0u;  // z <= tl
+                            m1 = nh ? ~a1 : 0u;  // z >= th
+                        }
+                        setn(pm, c, m0);
+                        setn(px, c, m1);
+                    }
+                    bool pend = (pm[0] | pm[1] | pm[2] | pm[3] | px[0] | px[1] | px[2] | px[3]) != 0;
+                    while (__any_sync(0xffffffffu, pend)) {
+                        const int cnt = __popc(pm[0] | px[0]) + __popc(pm[1] | px[1]) + __popc(pm[2] | px[2]) +
+                                        __popc(pm[3] | px[3]);
+                        int inc = cnt;
+#pragma unroll
+                        for (int off = 1; off < 32; off <<= 1) {
+                            const int t = __shfl_up_sync(0xffffffffu, inc, off);
+                            if (lane >= off) inc += t;
+                        }
+                        const int base = inc - cnt;
+                        const int total = __shfl_sync(0xffffffffu, inc, 31);
+                        int slot = base;
+#pragma unroll 1
+                        for (int c = 0; c < 4 && slot < kListCap; c++) {
+                            uint32_t m = pickn(pm, c) | pickn(px, c);
+                            while (m && slot < kListCap) {
+                                djobs[slot++] = (uint32_t)row | (uint32_t)(c * 32 + __ffs(m) - 1) << 8;
+                                m &= m - 1;
+                            }
+                        }
+                        __syncwarp();
+                        run_jobs<kJobSlots>(djobs, dres, min(total, kListCap), stg, Gf, g, lane);
+                        __syncwarp();
+                        slot = base;
+#pragma unroll 1
+                        for (int c = 0; c < 4 && slot < kListCap; c++) {
+                            const int bk = c / CPB;
+                            uint32_t cm = pickn(pm, c), cx = pickn(px, c);
+                            uint32_t m = cm | cx;
+                            float emn = pickn(ex_mn, bk), emx = pickn(ex_mx, bk);
+                            while (m && slot < kListCap) {
+                                const uint32_t bit = m & (0u - m);
+                                const float ze = dres[slot];
+                                if (cm & bit) emn = fminf(emn, ze);
+                                if (cx & bit) emx = fmaxf(emx, ze);
+                                cm &= ~bit;
+                                cx &= ~bit;
+                                m &= m - 1;
+                                slot++;
+                            }
+                            setn(ex_mn, bk, emn);
+                            setn(ex_mx, bk, emx);
+                            setn(pm, c, cm);
+                            setn(px, c, cx);
+                        }
+                        __syncwarp();
+                        pend = (pm[0] | pm[1] | pm[2] | pm[3] | px[0] | px[1] | px[2] | px[3]) != 0;
+                    }
+                } else {
+                    int nj = 0, c = 0;
+                    uint32_t todo = 0, left = 0xffffffffu;  // rows of chunk c to do; values of the first that no round has taken
+                    float tl, th;
+                    auto chunk_rows = [&]() -> uint32_t {  // rows with candidates in chunk c
+                        const int bk = c / CPB;
+                        const int need = (amb >> (2 * bk)) & 3;
+                        const float e2 = 2.0f * (TILE ? pickn(Et, bk) : bound(pickn(Ec, bk), pickn(mn, bk), pickn(mx, bk)));
+                        tl = __fadd_rn(pickn(mn, bk), e2);
+                        th = __fsub_rn(pickn(mx, bk), e2);
+                        // (tiles: a NaN z~ is a candidate, for which only the exact value can tell)
+                        const bool nl = need != 0 && (TILE ? !(pickn(cmn, c) > tl) : pickn(cmn, c) <= tl);
+                        const bool nh = (need & 1) && (TILE ? !(pickn(cmx, c) < th) : pickn(cmx, c) >= th);
+                        if (!nl) tl = -INFINITY;
+                        if (!nh) th = INFINITY;
+                        return __ballot_sync(0xffffffffu, nl || nh);
+                    };
+                    auto search = [&]() {  // appends the candidates of rows todo until the list is full
                         uint32_t v[32];
                         tmem_ld32(tacc + c * 32, v);
                         tmem_wait_ld();
@@ -578,21 +681,71 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                             todo &= todo - 1;
                             left = 0xffffffffu;
                         } while (todo);
-                        if (todo) flush();  // (the row's values need not survive it: they are loaded again)
+                    };
+                    auto flush = [&]() {
+                        __syncwarp();
+                        run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
+                        __syncwarp();
+#pragma unroll 1
+                        for (int j = 0; j < nj; j++) {
+                            const uint32_t w = jobs[j];
+                            const float ze = rowbuf[j];
+                            if ((int)(w & 31u) == lane) {
+                                const int bk = (int)((w >> 8) & 127u) / blk;
+                                if constexpr (kInPlace) {
+                                    if (bk != cur) {
+                                        if (cur >= 0) setn(sz, cur, exact(cur, pickn(sz, cur), ex_mn[0], ex_mx[0]));
+                                        cur = bk;
+                                        ex_mn[0] = INFINITY;
+                                        ex_mx[0] = -INFINITY;
+                                    }
+                                    if (w & 0x10000u) ex_mn[0] = fminf(ex_mn[0], ze);
+                                    if (w & 0x20000u) ex_mx[0] = fmaxf(ex_mx[0], ze);
+                                } else {
+                                    if (w & 0x10000u) setn(ex_mn, bk, fminf(pickn(ex_mn, bk), ze));
+                                    if (w & 0x20000u) setn(ex_mx, bk, fmaxf(pickn(ex_mx, bk), ze));
+                                }
+                            }
+                        }
+                        __syncwarp();
+                        nj = 0;
+                    };
+                    if constexpr (kOneSite) {
+                        do {
+#pragma unroll 1
+                            for (; c < 4; c++) {
+                                const uint32_t rows = chunk_rows();
+                                if (todo == 0) todo = rows;
+                                if (todo == 0) continue;
+                                search();
+                                if (todo) break;
+                            }
+                            if (nj) flush();
+                        } while (todo);
+                    } else {
+#pragma unroll 1
+                        for (; c < 4; c++) {
+                            todo = chunk_rows();
+                            while (todo) {
+                                search();
+                                if (todo) flush();  // (the row's values need not survive it: they are loaded again)
+                            }
+                        }
+                        if (nj) flush();
                     }
                 }
-                if (nj) flush();
+                if constexpr (kInPlace) {
+                    if (cur >= 0) setn(sz, cur, exact(cur, pickn(sz, cur), ex_mn[0], ex_mx[0]));
+                } else {
 #pragma unroll
-                for (int bk = 0; bk < NBK; bk++) {
-                    const int need = (amb >> (2 * bk)) & 3;
-                    if constexpr (TILE) {
-                        ex_mn[bk] = half_warp_min(ex_mn[bk]);
-                        ex_mx[bk] = half_warp_max(ex_mx[bk]);
-                        if ((need & 1) && ex_mn[bk] > ex_mx[bk]) ex_mn[bk] = ex_mx[bk] = NAN;  // no value but NaN
-                    }
-                    if (need) {
-                        m16[bk] = f2h_bits(ex_mn[bk]);
-                        if (need & 1) s16[bk] = scale16(ex_mx[bk], ex_mn[bk], qmaxf);
+                    for (int bk = 0; bk < NBK; bk++) {
+                        const int need = (amb >> (2 * bk)) & 3;
+                        if constexpr (TILE) {
+                            ex_mn[bk] = half_warp_min(ex_mn[bk]);
+                            ex_mx[bk] = half_warp_max(ex_mx[bk]);
+                            if ((need & 1) && ex_mn[bk] > ex_mx[bk]) ex_mn[bk] = ex_mx[bk] = NAN;  // no value but NaN
+                        }
+                        if (need) sz[bk] = exact(bk, sz[bk], ex_mn[bk], ex_mx[bk]);
                     }
                 }
             }
@@ -607,14 +760,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                 // a dead block (zero or overflowing scale) codes to 0 with r = c0 = 0, unless its z~ may not be
                 // finite: NaN takes the checked loop, whose clamp makes it 0
                 fast[bk] = Ec[bk] < INFINITY;
-                if (valid && (h_is_inf(s16[bk]) || h_is_inf(m16[bk]))) flag |= CG_FLAG_FP16_OVERFLOW;
-                const float sc = h2f_bits(s16[bk]), mz = h2f_bits(m16[bk]);
+                const uint32_t s16 = sz[bk] & 0xffffu, m16 = sz[bk] >> 16;
+                if (valid && (h_is_inf(s16) || h_is_inf(m16))) flag |= CG_FLAG_FP16_OVERFLOW;
+                const float sc = h2f_bits(s16), mz = h2f_bits(m16);
                 if constexpr (TILE) {
                     if (!fast[bk]) lim[bk] = -1.0f;  // no bound: every code of the row is recomputed
                     // the rule's code of a finite value over a zero of -inf: fl((z + inf) / s) clamps to qmax
-                    if (m16[bk] == 0xfc00u && sc != 0.0f && !h_is_inf(s16[bk])) c0[bk] = qmaxf;
+                    if (m16 == 0xfc00u && sc != 0.0f && !h_is_inf(s16)) c0[bk] = qmaxf;
                 }
-                if (sc != 0.0f && !h_is_inf(s16[bk]) && !h_is_inf(m16[bk])) {
+                if (sc != 0.0f && !h_is_inf(s16) && !h_is_inf(m16)) {
                     const float r = __frcp_rn(sc);
                     const float cc = -mz * r;
                     rinv[bk] = r;
@@ -627,7 +781,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     // every code is the exact rule's)
                     // (fmaxf: without a bound every code)
                     lim[bk] = TILE ? fmaxf(0.5f - mu, -1.0f) : (mu < 0.99e-4f ? 2.0f : 0.5f - mu);
-                    const float tlo = (mn[bk] - E[bk]) * r + cc, thi = (mx[bk] + E[bk]) * r + cc;
+                    const float e = TILE ? Et[TILE ? bk : 0] : bound(Ec[bk], mn[bk], mx[bk]);
+                    const float tlo = (mn[bk] - e) * r + cc, thi = (mx[bk] + e) * r + cc;
                     fast[bk] = tlo > -0.49f + mu && thi < qmaxf + 0.49f - mu && (kTrack || lim[bk] > 1.0f);
                 }
             }
@@ -635,6 +790,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
             // ---- 6. codes from z~, stored straight from registers
             uint8_t* crow = a.codes + a.cmap.at(ti.l, ti.s, ti.b, ti.h, ti.t0 + row);
             int nj = 0;  // values within mu of a rounding boundary, to be recomputed exactly and patched
+            uint32_t am[4] = {0, 0, 0, 0};  // (MASKS: as masks)
             auto patch = [&]() {
                 __syncwarp();
                 run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
@@ -645,7 +801,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     const float ze = rowbuf[j];
                     if ((int)(w & 31u) == lane) {
                         const int col = (int)((w >> 8) & 127u), bk = col / blk;
-                        patch_code<BITS>(crow, col * BITS, quant_code(ze, h2f_bits(pickn(s16, bk)), h2f_bits(pickn(m16, bk)), qmax));
+                        patch_code<BITS>(crow, col * BITS, quant_code(ze, h2f_bits(pickn(sz, bk) & 0xffffu), h2f_bits(pickn(sz, bk) >> 16), qmax));
                     }
                 }
                 __syncwarp();
@@ -663,6 +819,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
 #pragma unroll
                 for (int w = 0; w < BITS; w++) words[w] = 0;
                 float worst = 0.0f;  // the largest distance from an integer of this lane's values
+                uint32_t mk = 0;     // or a mask of those beyond lm
                 const float2 r2 = make_float2(r, r), c2 = make_float2(cz, cz), m2 = make_float2(kMagic, kMagic);
                 const float2 n2 = make_float2(-kMagic, -kMagic);
                 if (__all_sync(0xffffffffu, TILE ? fst || !valid : fst)) {
@@ -679,6 +836,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                             worst = max3f(worst, fabsf(e.x), fabsf(e.y));
                         }
                     }
+                } else if constexpr (MASKS) {  // the same codes; values beyond lm as a mask
+                    const float lm = pickn(lim, bk);
+#pragma unroll
+                    for (int k = 31; k >= 0; k--) {
+                        float t = fmaf(__uint_as_float(v[k]), r, cz);
+                        t = fminf(fmaxf(t, 0.0f), qmaxf);
+                        const float y = t + kMagic;
+                        mk = __funnelshift_l(__float_as_uint(__fsub_rn(lm, fabsf(t - (y - kMagic)))), mk, 1);
+                        put_code<BITS>(words, k, __float_as_uint(y));
+                    }
+                    if (fst) mk = 0;
                 } else {
                     // clamping before the rounding gives the same code as clamping after it
 #pragma unroll
@@ -711,10 +879,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                     }
                 }
                 // ---- 7. values within mu of a rounding boundary: exact recompute and patch
+                if constexpr (MASKS) {
+                    if (valid) setn(am, c, mk);
+                    continue;
+                }
                 const float lm = pickn(lim, bk);
-                uint32_t todo = __ballot_sync(0xffffffffu, valid && worst > lm);
-                uint32_t left = 0xffffffffu;
-                while (todo) {
+                uint32_t todo = __ballot_sync(0xffffffffu, valid && worst > lm), left = 0xffffffffu;
+                auto search = [&]() {  // appends the marked values of rows todo until the list is full
                     tmem_ld32(tacc + c * 32, v);
                     tmem_wait_ld();
                     do {
@@ -729,24 +900,77 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
                         todo &= todo - 1;
                         left = 0xffffffffu;
                     } while (todo);
-                    if (todo) patch();
+                };
+                if constexpr (kOneSite) {
+                    while (todo || (c == 3 && nj)) {
+                        if (todo) search();
+                        if (!todo && c < 3) break;
+                        patch();
+                    }
+                } else {
+                    while (todo) {
+                        search();
+                        if (todo) patch();
+                    }
                 }
             }
-            if (nj) patch();
+            if constexpr (!kOneSite && !MASKS) {
+                if (nj) patch();
+            }
+            if constexpr (MASKS) {
+                bool pend = (am[0] | am[1] | am[2] | am[3]) != 0;
+                while (__any_sync(0xffffffffu, pend)) {
+                    const int cnt = __popc(am[0]) + __popc(am[1]) + __popc(am[2]) + __popc(am[3]);
+                    int inc = cnt;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const int t = __shfl_up_sync(0xffffffffu, inc, off);
+                        if (lane >= off) inc += t;
+                    }
+                    const int base = inc - cnt;
+                    const int total = __shfl_sync(0xffffffffu, inc, 31);
+                    int slot = base;
+#pragma unroll 1
+                    for (int c = 0; c < 4 && slot < kListCap; c++) {
+                        uint32_t m = pickn(am, c);
+                        while (m && slot < kListCap) {
+                            djobs[slot++] = (uint32_t)row | (uint32_t)(c * 32 + __ffs(m) - 1) << 8;
+                            m &= m - 1;
+                        }
+                    }
+                    __syncwarp();
+                    run_jobs<kJobSlots>(djobs, dres, min(total, kListCap), stg, Gf, g, lane);
+                    __syncwarp();
+                    slot = base;
+#pragma unroll 1
+                    for (int c = 0; c < 4 && slot < kListCap; c++) {
+                        const int bk = c / CPB;
+                        uint32_t m = pickn(am, c);
+                        const float sb = h2f_bits(pickn(sz, bk) & 0xffffu), mb = h2f_bits(pickn(sz, bk) >> 16);
+                        while (m && slot < kListCap) {
+                            const int col = c * 32 + __ffs(m) - 1;
+                            patch_code<BITS>(crow, col * BITS, quant_code(dres[slot], sb, mb, qmax));
+                            m &= m - 1;
+                            slot++;
+                        }
+                        setn(am, c, m);
+                    }
+                    __syncwarp();
+                    pend = (am[0] | am[1] | am[2] | am[3]) != 0;
+                }
+            }
 
             // ---- 8. scales (tiles: one set for the 16 rows); release the stage and the accumulator
             if (valid && (!TILE || (row & (CG_TILE_TOKENS - 1)) == 0)) {
                 uint32_t* sp = a.scales + a.smap.at(ti.l, ti.s, ti.b, ti.h, ti.t0 + row);
                 const bool vec = (reinterpret_cast<uintptr_t>(sp) & (NBK * 4 - 1)) == 0;
                 if (NBK == 4 && vec) {
-                    *reinterpret_cast<uint4*>(sp) = make_uint4(s16[0] | (m16[0] << 16), s16[1] | (m16[1] << 16),
-                                                               s16[NBK > 2 ? 2 : 0] | (m16[NBK > 2 ? 2 : 0] << 16),
-                                                               s16[NBK > 3 ? 3 : 0] | (m16[NBK > 3 ? 3 : 0] << 16));
+                    *reinterpret_cast<uint4*>(sp) = make_uint4(sz[0], sz[NBK > 1 ? 1 : 0], sz[NBK > 2 ? 2 : 0], sz[NBK > 3 ? 3 : 0]);
                 } else if (NBK == 2 && vec) {
-                    *reinterpret_cast<uint2*>(sp) = make_uint2(s16[0] | (m16[0] << 16), s16[NBK > 1 ? 1 : 0] | (m16[NBK > 1 ? 1 : 0] << 16));
+                    *reinterpret_cast<uint2*>(sp) = make_uint2(sz[0], sz[NBK > 1 ? 1 : 0]);
                 } else {
 #pragma unroll
-                    for (int bk = 0; bk < NBK; bk++) sp[bk] = s16[bk] | (m16[bk] << 16);
+                    for (int bk = 0; bk < NBK; bk++) sp[bk] = sz[bk];
                 }
             }
             tc_fence_before();
@@ -767,22 +991,41 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
     }
 }
 
-template <int BITS, int NBK, bool TILE>
+template <int BITS, int NBK, bool TILE, bool MASKS>
 cudaError_t launch_rows(const RowEncParams& P, const CUtensorMap& map, cudaStream_t st) {
     const size_t smem = RowSmem::total;
-    cudaError_t e = cudaFuncSetAttribute(tc_rows_encode_kernel<BITS, NBK, TILE>,
+    cudaError_t e = cudaFuncSetAttribute(tc_rows_encode_kernel<BITS, NBK, TILE, MASKS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = P.S.n_tiles < tc::num_sms() ? P.S.n_tiles : tc::num_sms();
-    tc_rows_encode_kernel<BITS, NBK, TILE><<<(unsigned)grid, kThreads, smem, st>>>(map, P);
+    tc_rows_encode_kernel<BITS, NBK, TILE, MASKS><<<(unsigned)grid, kThreads, smem, st>>>(map, P);
     return cudaGetLastError();
 }
 
 template <int BITS, bool TILE>
 cudaError_t launch_rows_bits(const RowEncParams& P, const CUtensorMap& map, cudaStream_t st) {
-    if (P.a.blk == 128) return launch_rows<BITS, 1, TILE>(P, map, st);
-    if (P.a.blk == 64) return launch_rows<BITS, 2, TILE>(P, map, st);
-    return launch_rows<BITS, 4, TILE>(P, map, st);
+    // Masks or search (kernel time, masks / search; a CTA per SM, so tiles / SMs is a CTA's tiles):
+    // 32-channel blocks: g = 128 119 / 128 us (27 tiles a CTA, 4 bits), 22.1 / 24.9 (1 tile); g = 64
+    // 100 / 99 and 16.5 / 19.6; g = 32 94 / 90, 21.6 / 21.8 (3 tiles) and 15.3 / 16.5 (1 tile).
+    // 64 channels, g = 128, 1 to 4 tiles: 24.4 / 25.0 us (4 bits), 28.9 / 29.6; at 7 tiles 37.9 / 38.3.
+    // 8 bits, 64 or 128 channels, g >= 64 (many codes near a rounding boundary): 21.8 / 23.0 us at 1
+    // tile, 46.2 / 48.2 at 7, 127 / 120 at 27; below g = 64 only at one tile (14.0 / 15.6 us).
+    const int64_t sms = tc::num_sms(), tiles = P.S.n_tiles;
+    const int g = P.a.g;
+    if constexpr (!TILE) {
+        const bool few = tiles <= 4 * sms;
+        if (P.a.blk == 32 && (g == 128 || few)) return launch_rows<BITS, 4, TILE, true>(P, map, st);
+        if constexpr (BITS == 8) {
+            const bool masks = tiles <= (g >= 64 ? 8 : 1) * sms;
+            if (P.a.blk == 64 && masks && g >= 64) return launch_rows<BITS, 2, TILE, true>(P, map, st);
+            if (P.a.blk == 128 && masks) return launch_rows<BITS, 1, TILE, true>(P, map, st);
+        } else {
+            if (P.a.blk == 64 && g == 128 && few) return launch_rows<BITS, 2, TILE, true>(P, map, st);
+        }
+    }
+    if (P.a.blk == 128) return launch_rows<BITS, 1, TILE, false>(P, map, st);
+    if (P.a.blk == 64) return launch_rows<BITS, 2, TILE, false>(P, map, st);
+    return launch_rows<BITS, 4, TILE, false>(P, map, st);
 }
 
 template <bool TILE>
