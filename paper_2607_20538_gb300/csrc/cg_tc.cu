@@ -18,7 +18,9 @@
 // heads of 32k tokens at 3 bits, keys and values). The candidates of an undecided range and
 // the values near a rounding boundary are found by spreading a channel's 32 values over the
 // lanes (one compare and vote) instead of by masks in every lane, and codes are made in
-// packed pairs: 4.49 -> 3.89 ms.
+// packed pairs: 4.49 -> 3.89 ms; the exact rounds at one call site each: 3.85 ms. Where a CTA
+// has few tiles nothing hides the chain of that search, and the extremes are looked for by
+// masks (MASKS; launch_encode_bits).
 //
 // Exactness. The library defines z as a fixed-order fp32 sum (pairwise summation of the
 // products; include/codecgauge.h). For every output channel i the converter bounds
@@ -83,7 +85,7 @@ struct Misc {
     uint32_t tmem_slot;
     int abort_flag;
     float emaxb[kSegBufs][4];  // per gauge set and quantization block: max_i e_i
-    float gmaxb[kSegBufs][4];  // and max_i ||G_i||
+    float gmaxb[kSegBufs][4];  // and max_i ||G_i|| (the converter's, not read here)
     uint64_t xbar[3][2];       // keys: per warpgroup, exchange of the group-norm maxima
 };
 
@@ -153,7 +155,7 @@ __device__ __forceinline__ void patch_code(uint8_t* rowp, int bit, uint32_t q) {
 
 // The MMA's operands are swapped against the row kernel's, D[channel][token] = G x^T, so a
 // thread owns one channel's 128 tokens, which form its block and its packed code stream.
-template <int BITS, bool KEYS, int NBK>
+template <int BITS, bool KEYS, int NBK, bool MASKS>
 __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_constant__ CUtensorMap xmap,
                                                                  const EncParams P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -485,34 +487,51 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
             if (__any_sync(0xffffffffu, amb != 0)) {
                 const int need = amb & 3;
                 float ex_mn = INFINITY, ex_mx = -INFINITY;
-                int nj = 0;
-                auto flush = [&]() {
-                    __syncwarp();
-                    tce::run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
-                    __syncwarp();
-#pragma unroll 1
-                    for (int j = 0; j < nj; j++) {
-                        const uint32_t w = jobs[j];
-                        const float ze = rowbuf[j];
-                        if ((int)((w >> 8) & 31u) == lane) {
-                            if (w & 0x10000u) ex_mn = fminf(ex_mn, ze);
-                            if (w & 0x20000u) ex_mx = fmaxf(ex_mx, ze);
-                        }
-                    }
-                    __syncwarp();
-                    nj = 0;
-                };
+                uint32_t m0 = 0, m1 = 0;  // MASKS: candidates of this lane's channel in chunk c, once made
+                bool made = false;
+                int nj = 0, c = 0;
+                uint32_t todo = 0, left = 0xffffffffu;  // channels of chunk c to do; values of the first that no round has taken
                 const float e2 = 2.0f * E[0], tl0 = __fadd_rn(mn[0], e2), th0 = __fsub_rn(mx[0], e2);
+                do {
 #pragma unroll 1
-                for (int c = 0; c < 4; c++) {
-                    const bool nl = need != 0 && !(pick4(cmn, c) > tl0);  // a NaN z~ is a candidate
-                    const bool nh = (need & 1) && !(pick4(cmx, c) < th0);
-                    uint32_t todo = __ballot_sync(0xffffffffu, nl || nh);
-                    if (todo == 0) continue;
-                    const float tl = nl ? tl0 : -INFINITY, th = nh ? th0 : INFINITY;
-                    uint32_t left = 0xffffffffu;  // values of channel src that no earlier round has taken
-                    while (todo) {
+                    for (; c < 4; c++) {
+                        const bool nl = need != 0 && !(pick4(cmn, c) > tl0);  // a NaN z~ is a candidate
+                        const bool nh = (need & 1) && !(pick4(cmx, c) < th0);
+                        if (todo == 0) todo = __ballot_sync(0xffffffffu, nl || nh);
+                        if (todo == 0) continue;
+                        const float tl = nl ? tl0 : -INFINITY, th = nh ? th0 : INFINITY;
                         uint32_t v[32];
+                        if constexpr (MASKS) {
+                            if (!made) {
+                                tmem_ld32(tacc + c * 32, v);
+                                tmem_wait_ld();
+                                uint32_t a0 = 0, a1 = 0;  // sign bits of tl0 - z (z > tl0) and z - th0 (z < th0)
+#pragma unroll
+                                for (int k = 31; k >= 0; k--) {
+                                    const float z = __uint_as_float(v[k]);
+                                    a0 = __funnelshift_l(__float_as_uint(__fsub_rn(tl0, z)), a0, 1);
+                                    a1 = __funnelshift_l(__float_as_uint(__fsub_rn(z, th0)), a1, 1);
+                                }
+                                m0 = nl ? ~a0 : 0u;
+                                m1 = nh ? ~a1 : 0u;
+                                made = true;
+                            }
+                            do {
+                                const uint32_t m = m0 | m1, bit = m & (0u - m);
+                                todo = __ballot_sync(0xffffffffu, m != 0);
+                                if (!todo) break;
+                                const uint32_t word = (uint32_t)(c * 32 + __ffs(m) - 1) | (uint32_t)row << 8 |
+                                                      ((m0 & bit) ? 0x10000u : 0u) | ((m1 & bit) ? 0x20000u : 0u);
+                                left = append(jobs, kJobCap, todo, word, nj);
+                                if (!((left >> lane) & 1u)) {
+                                    m0 &= ~bit;
+                                    m1 &= ~bit;
+                                }
+                            } while (!left);
+                            if (todo) break;  // the list is full
+                            made = false;
+                            continue;
+                        }
                         tmem_ld32(tacc + c * 32, v);
                         tmem_wait_ld();
                         do {
@@ -526,10 +545,25 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
                             todo &= todo - 1;
                             left = 0xffffffffu;
                         } while (todo);
-                        if (todo) flush();  // (the values need not survive it: they are loaded again)
+                        if (todo) break;
                     }
-                }
-                if (nj) flush();
+                    if (nj) {
+                        __syncwarp();
+                        tce::run_jobs<kJobSlots>(jobs, rowbuf, nj, stg, Gf, g, lane);
+                        __syncwarp();
+#pragma unroll 1
+                        for (int j = 0; j < nj; j++) {
+                            const uint32_t w = jobs[j];
+                            const float ze = rowbuf[j];
+                            if ((int)((w >> 8) & 31u) == lane) {
+                                if (w & 0x10000u) ex_mn = fminf(ex_mn, ze);
+                                if (w & 0x20000u) ex_mx = fmaxf(ex_mx, ze);
+                            }
+                        }
+                        __syncwarp();
+                        nj = 0;
+                    }
+                } while (todo);
                 if (need) {
                     m16[0] = f2h_bits(ex_mn);
                     if (need & 1) s16[0] = scale16(ex_mx, ex_mn, qmaxf);
@@ -573,20 +607,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
             constexpr int kCodeCap = kMasks ? (32 + kJobCap) / 2 : kJobCap;
             uint32_t* cjobs = kMasks ? reinterpret_cast<uint32_t*>(rowbuf) : jobs;
             float* cres = kMasks ? rowbuf + kCodeCap : rowbuf;
-            auto patch = [&]() {
-                __syncwarp();
-                tce::run_jobs<kJobSlots>(cjobs, cres, nj, stg, Gf, g, lane);
-                __syncwarp();
-#pragma unroll 1
-                for (int j = 0; j < nj; j++) {
-                    const uint32_t w = cjobs[j];
-                    const float ze = cres[j];
-                    if ((int)((w >> 8) & 31u) == lane)
-                        patch_code<BITS>(crow, (int)(w & 127u) * BITS, quant_code(ze, h2f_bits(s16[0]), h2f_bits(m16[0]), qmax));
-                }
-                __syncwarp();
-                nj = 0;
-            };
             const float r = rinv[0], cc = c0[0], lm = lim[0];
 #pragma unroll 1
             for (int c = 0; c < 4; c++) {
@@ -639,36 +659,48 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
 #pragma unroll
                     for (int w = 0; w < BITS; w++) dst[w] = words[w];
                 }
-                if constexpr (kMasks) {
-                    while (__any_sync(0xffffffffu, mask != 0)) {
-                        const uint32_t word = (uint32_t)(c * 32 + __ffs(mask) - 1) | (uint32_t)row << 8;
-                        const uint32_t left = append(cjobs, kCodeCap, __ballot_sync(0xffffffffu, mask != 0), word, nj);
-                        if (!((left >> lane) & 1u)) mask &= mask - 1;
-                        if (left) patch();  // the list is full
+                uint32_t todo = __ballot_sync(0xffffffffu, kMasks ? mask != 0 : worst > lm), left = 0xffffffffu;
+                while (todo || (c == 3 && nj)) {
+                    if (todo) {
+                        if constexpr (kMasks) {
+                            do {
+                                const uint32_t word = (uint32_t)(c * 32 + __ffs(mask) - 1) | (uint32_t)row << 8;
+                                left = append(cjobs, kCodeCap, todo, word, nj);
+                                if (!((left >> lane) & 1u)) mask &= mask - 1;
+                                todo = __ballot_sync(0xffffffffu, mask != 0);
+                            } while (todo && !left);
+                        } else {
+                            tmem_ld32(tacc + c * 32, v);
+                            tmem_wait_ld();
+                            do {
+                                const int src = __ffs(todo) - 1;
+                                const float sr = __shfl_sync(0xffffffffu, r, src), sc = __shfl_sync(0xffffffffu, cc, src);
+                                const float sl = __shfl_sync(0xffffffffu, lm, src);
+                                const float z = spread(v, src);
+                                const float t = fminf(fmaxf(fmaf(z, sr, sc), 0.0f), qmaxf);
+                                left = append(cjobs, kCodeCap, __ballot_sync(0xffffffffu, fabsf(t - ((t + kMagic) - kMagic)) > sl) & left,
+                                              (uint32_t)(c * 32 + lane) | (uint32_t)(q4 * 32 + src) << 8, nj);
+                                if (left) break;  // the list is full
+                                todo &= todo - 1;
+                                left = 0xffffffffu;
+                            } while (todo);
+                        }
+                        if (!todo && c < 3) break;
                     }
-                } else {
-                    uint32_t todo = __ballot_sync(0xffffffffu, worst > lm);
-                    uint32_t left = 0xffffffffu;
-                    while (todo) {
-                        tmem_ld32(tacc + c * 32, v);
-                        tmem_wait_ld();
-                        do {
-                            const int src = __ffs(todo) - 1;
-                            const float sr = __shfl_sync(0xffffffffu, r, src), sc = __shfl_sync(0xffffffffu, cc, src);
-                            const float sl = __shfl_sync(0xffffffffu, lm, src);
-                            const float z = spread(v, src);
-                            const float t = fminf(fmaxf(fmaf(z, sr, sc), 0.0f), qmaxf);
-                            left = append(cjobs, kCodeCap, __ballot_sync(0xffffffffu, fabsf(t - ((t + kMagic) - kMagic)) > sl) & left,
-                                          (uint32_t)(c * 32 + lane) | (uint32_t)(q4 * 32 + src) << 8, nj);
-                            if (left) break;  // the list is full
-                            todo &= todo - 1;
-                            left = 0xffffffffu;
-                        } while (todo);
-                        if (todo) patch();
+                    __syncwarp();
+                    tce::run_jobs<kJobSlots>(cjobs, cres, nj, stg, Gf, g, lane);
+                    __syncwarp();
+#pragma unroll 1
+                    for (int j = 0; j < nj; j++) {
+                        const uint32_t w = cjobs[j];
+                        const float ze = cres[j];
+                        if ((int)((w >> 8) & 31u) == lane)
+                            patch_code<BITS>(crow, (int)(w & 127u) * BITS, quant_code(ze, h2f_bits(s16[0]), h2f_bits(m16[0]), qmax));
                     }
+                    __syncwarp();
+                    nj = 0;
                 }
             }
-            if (nj) patch();
 
             // ---- 7. scales; release the stage and the accumulator buffer
             if (valid) {
@@ -696,14 +728,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_encode_kernel(const __grid_con
     }
 }
 
-template <int BITS, bool KEYS, int NBK>
+template <int BITS, bool KEYS, int NBK, bool MASKS>
 cudaError_t launch_encode_nbk(const EncParams& P, const CUtensorMap& map, cudaStream_t st) {
     const size_t smem = EncSmem::total;
     cudaError_t e =
-        cudaFuncSetAttribute(tc_encode_kernel<BITS, KEYS, NBK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(tc_encode_kernel<BITS, KEYS, NBK, MASKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = P.S.n_tiles < tc::num_sms() ? P.S.n_tiles : tc::num_sms();
-    tc_encode_kernel<BITS, KEYS, NBK><<<(unsigned)grid, kThreads, smem, st>>>(map, P);
+    tc_encode_kernel<BITS, KEYS, NBK, MASKS><<<(unsigned)grid, kThreads, smem, st>>>(map, P);
     return cudaGetLastError();
 }
 
@@ -712,7 +744,10 @@ cudaError_t launch_encode_nbk(const EncParams& P, const CUtensorMap& map, cudaSt
 template <int BITS, bool KEYS>
 cudaError_t launch_encode_bits(const EncParams& P, const CUtensorMap& map, cudaStream_t st) {
     static_assert(KEYS, "rows are encoded by tc_rows_encode_kernel");
-    return launch_encode_nbk<BITS, KEYS, 1>(P, map, st);
+    // one tile a CTA, masks / search: 24.2 / 25.1 us (2 bits, g = 128), 20.8 / 22.1 (6 bits, g = 64), 16.3 / 16.2 (4
+    // bits, g = 32); 13 tiles: 95.9 / 93.2 us (keys and values, 2 bits, g = 32), 139.6 / 136.5 (6 bits, g = 64)
+    if (P.S.n_tiles <= 4 * (int64_t)tc::num_sms()) return launch_encode_nbk<BITS, KEYS, 1, true>(P, map, st);
+    return launch_encode_nbk<BITS, KEYS, 1, false>(P, map, st);
 }
 
 template <bool KEYS>

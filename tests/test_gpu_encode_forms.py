@@ -33,3 +33,11 @@ def test_rows(bits, group, block, per_sm, over):
     B = per_sm * sms // 8 + over  # 8 units a sequence
     w = synth.Workload("forms", L=1, B=B, H=4, T=70, d=128, group=group, backend=0, bits=bits, block=block, residual=0)
     _run(w, _inputs(w), synth.gauges(w))
+
+
+@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("bits,group", [(2, 32), (3, 128), (4, 64), (6, 64), (8, 128)])
+def test_keys(bits, group, over):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = synth.Workload("forms", L=1, B=sms + over, H=4, T=130, d=128, group=group, backend=1, bits=bits, block=128, residual=2)
+    _run(w, _inputs(w), synth.gauges(w))
