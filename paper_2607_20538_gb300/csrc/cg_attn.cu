@@ -403,12 +403,12 @@ __global__ void __launch_bounds__(SL * kAD) attn_combine_kernel(AttnArgs a) {
 // blocks per row, 7.5 of them unpacking; 87 in the kernel it replaced, whose value sums ran on CUDA
 // cores; with the queries as the 16-row operand instead, twice the MMAs for four queries, 308 us
 // against 298). One layer, 64 sequences x 8 heads x 16,384 tokens, 4 bits, 4 queries a head: whole
-// call 1043 -> 281 us (stream kernel 255 us, 4.7 TB/s, 70 % of measured HBM); one 32,767-token
-// sequence at 8 bits 280 -> 43 us.
+// call 1043 -> 268 us (stream kernel 242 us, 5.0 TB/s, 73 % of measured HBM); one 32,767-token
+// sequence at 8 bits 280 -> 42 us.
 // ------------------------------------------------------------------------------------
 constexpr int kSThreads = 128;
 constexpr int kSWarps = kSThreads / 32;
-constexpr int kSCtas = 3;  // per SM: 168 registers a thread; four CTAs (128 registers) spill
+constexpr int kSCtas = 3;  // per SM: 168 registers a thread, up to 46 bytes spilled (2 bits, four blocks, eight queries); four CTAs (128 registers) spill far more
 
 template <int BITS, int NB>
 struct StreamCfg {
@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(kSThreads, kSCtas) attn_stream_kernel(AttnArgs
         for (int off = 1; off < 4; off <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
         // scaled by the power of two that takes the largest value into [2^14, 2^15)
         int E = (int)(__float_as_uint(amax) >> 23);
-        E = E < 20 ? 20 : (E > 230 ? 230 : E);
+        E = E < 20 ? 20 : (E > 254 ? 254 : E);
         const float up = __uint_as_float((uint32_t)(268 - E) << 23);
         if (warp == 0 && t == 0 && (Q8 || g < 4)) {
             float* st = stat + qi * (2 * NB + 1);
@@ -622,7 +622,8 @@ __global__ void __launch_bounds__(kSThreads, kSCtas) attn_stream_kernel(AttnArgs
                 st[2 * k] = c1[k] * up * 5.9604645e-08f;
                 st[2 * k + 1] = kOff * c2[k] * up * 5.9604645e-08f;
             }
-            st[2 * NB] = __uint_as_float((uint32_t)(E + 10) << 23) * kLog2e;
+            // (at most 2^126: score differences beyond 2^102 leave a weight of 0 either way)
+            st[2 * NB] = __uint_as_float((uint32_t)(E < 243 ? E + 10 : 253) << 23) * kLog2e;
         }
         for (int s = 2 * warp; s < 2 * warp + 2; s++) {  // two of the eight MMA steps per warp
             const int k = s / kKs, ks = s % kKs;
@@ -676,7 +677,7 @@ __global__ void __launch_bounds__(kSThreads, kSCtas) attn_stream_kernel(AttnArgs
         // off by at most 2^-23 of it or 2^-39 of that scale, whatever the scales of other steps are. The
         // sums follow by an exact power of two. (A factor from a stream's first step only, dropped when a
         // weight overflowed: up to 280 times the tests' tolerance after a prefix of zero scales; this rule
-        // takes the same time or less, 62.5 -> 59.5 us for 32 x 8 x 4,000 tokens at 4 bits in one block.)
+        // takes the same time or less, 62.5 -> 59.4 us for 32 x 8 x 4,000 tokens at 4 bits in one block.)
         int top = 0;
 #pragma unroll
         for (int e = 0; e < kItems; e++) {
@@ -807,13 +808,15 @@ __global__ void __launch_bounds__(kSThreads, kSCtas) attn_stream_kernel(AttnArgs
         const float2 al = make_float2(ex2((Mu.x - m.x) * cF.x), ex2((Mu.y - m.y) * cF.y));  // 0 on the first step
         const float2 al_acc = make_float2(al.x * rescale, al.y * rescale);
         Mu = m;
-        const float2 bias = make_float2(-m.x * cF.x, -m.y * cF.y);
+        const float2 neg = make_float2(-m.x, -m.y);
         float2 l2 = dup(0.0f);
 #pragma unroll
         for (int j = 0; j < kTiles; j++)
 #pragma unroll
             for (int hf = 0; hf < 2; hf++) {
-                const float2 e = __ffma2_rn(S[j][hf], cF, bias);
+                // the difference first: it is exact near the maximum and never above 0, however large the scores
+                // are (S cF less a rounded m cF is off by 2^-24 of it: NaN from scores of 2^23 on)
+                const float2 e = __fmul2_rn(__fadd2_rn(S[j][hf], neg), cF);
                 S[j][hf] = make_float2(ex2(e.x), ex2(e.y));
                 l2 = __fadd2_rn(l2, S[j][hf]);
             }

@@ -6,10 +6,12 @@ tokens hold: a prefix without values (zero padding), with tiny ones, or scales t
 history. 512 units, so that a warp streams through whole histories. Reference and tolerance as in
 test_gpu_attention.py, relative to the largest value of a unit; queries of standard deviation 1 at 2
 and 4 bits, the inputs that tolerance was derived for, and 2 at 8 bits, whose queries are not rounded.
+Queries up to the largest bf16 values: the scores' differences decide, however large they are.
 """
 import numpy as np
 import pytest
 
+import oracle
 from paper_2607_20538_gb300 import synth
 
 from test_gpu_attention import _run, _wl
@@ -54,3 +56,15 @@ def test_scales_that_drift(bits, block, grow):
     """Fourteen octaves over the history."""
     f = 2.0 ** -np.floor(np.linspace(0.0, 14.99, T))
     _check(bits, 4, f[::-1] if grow else f, block)
+
+
+@pytest.mark.parametrize("bits,n_rep,block", [(2, 8, 32), (4, 4, 64), (8, 1, 128), (8, 8, 64)])
+@pytest.mark.parametrize("size", [1.0e7, 1.0e20, 1.0e37])
+def test_large_queries(bits, n_rep, block, size):
+    """Scores of any fp32 size: the largest takes all the weight."""
+    w = _wl(L=1, B=2, H=2, T=300, bits=bits, block=block, group=32)
+    ref = oracle.encode(w.shape, w.params, synth.kv_cache(w, threads=4), synth.gauges(w))
+    q = size * np.random.default_rng(9).normal(0.0, 1.0, (w.L, w.B, w.H, n_rep, w.d))
+    dc = torch.from_numpy(np.concatenate([ref["codes"], np.zeros(16, np.uint8)])).cuda()
+    ds = torch.from_numpy(np.concatenate([ref["scales"], np.zeros(8, np.uint16)]).view(np.int16)).cuda()
+    _run(w, n_rep, 0, w.T, dc, ds, ref["codes"], ref["scales"], synth.gauges(w), synth.f32_to_bf16_bits(q.astype(np.float32)))
