@@ -224,12 +224,19 @@ int cg_kivi_stream_decode(const cg_shape* shape, const cg_params* params, const 
  * over tokens [t0, t0 + T) of the cache, where khat, vhat are what cg_decode would recover.
  * The inverse gauge is folded out of the token loop: q is rotated once into gauge space
  * (q . G^T zhat = (G q) . zhat) and the weighted sum of values stays in gauge space until one
- * G_V^T per query, so the kernels read only codes and scales. Arithmetic is fp32 (scores,
- * softmax, sums); the result is fp32, not bit-exact (see the tolerance in the tests).
+ * G_V^T per query, so the kernels read only codes and scales. Scores, softmax and sums are kept
+ * in fp32. At 2, 4 and 8 bits the two contractions run on tensor cores: the codes enter exactly,
+ * the rotated query (at 2 and 4 bits its bf16 pair and a quarter of the rest) and the weights
+ * p_t s_t as fp16 high and low parts (off by at most 2^-23 of the value; a weight by 2^-39 of the
+ * largest scale among the 32 or 64 tokens of its step where that is more), and the fp32
+ * accumulator of an MMA chain covers at most 64 tokens. The result is fp32, not bit-exact (see
+ * the tolerance in the tests): the tokens of a sequence are summed in parts that depend on the
+ * call's shape and on the sequence's place in it, so equal sequences of one call may differ in
+ * the last bits. Two calls with the same arguments give the same bits.
  * Supported: CG_BLOCK_UNIFORM and CG_BLOCK_TILE caches with d = 128 and block in {32, 64, 128},
  * any group and bit width; n_rep in {1, 2, 4, 8}; T >= 1. q: bf16 [L][B][H][n_rep][d];
  * out: fp32 [L][B][H][n_rep][d]. workspace: caller-owned device scratch of
- * cg_attention_workspace_bytes (rotated queries and per-512-token partial results). */
+ * cg_attention_workspace_bytes (rotated queries and partial results, room for one per 128 tokens). */
 int cg_attention_workspace_bytes(const cg_shape* shape, const cg_params* params, int n_rep,
                                  size_t* workspace_bytes);
 
