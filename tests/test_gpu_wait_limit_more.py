@@ -1,10 +1,11 @@
 """Bounded waits of the attention stream, the tile encoder and the Hadamard encoder; attention in a graph.
 
-As in test_gpu_wait_limit.py: with a limit of 100 ns the encoders' first copy cannot land in time, so
-the call comes back with CG_FLAG_PIPE_TIMEOUT and without any fault, and the next call, with the
-normal limit, gives the bytes that a call before gave. Attention starts its copies well before it waits
-for them, so it may not run out; without the flag its result has to be the right one. Shares that span
-several units and units of several parts. Its kernels are chained by programmatic launches, so a
+As in test_gpu_wait_limit.py: with a limit of 100 ns the tile encoder's first waits (for the gauge's
+conversion) cannot be met, so the call comes back with CG_FLAG_PIPE_TIMEOUT and without any fault, and
+the next call, with the normal limit, gives the bytes that a call before gave. The Hadamard encoder
+waits for one copy only, which may land between two ticks of the clock that the limit is read from, and
+attention starts its copies well before it waits for them: these may not run out, and without the flag
+the result has to be the right one. Shares that span several units and units of several parts. Its kernels are chained by programmatic launches, so a
 captured call is replayed on other inputs and compared with a plain call.
 """
 import numpy as np
@@ -51,7 +52,7 @@ def test_encoders(hadamard, monkeypatch):
     x, G = _cache(w)
     codes, scales, _ = cg.alloc_outputs(shape, params)
     call = (lambda: cg.encode_hadamard(shape, params, x, codes, scales)) if hadamard else (lambda: cg.encode(shape, params, x, G, codes, scales))
-    _timeout_then_same(call, [codes, scales], monkeypatch)
+    _timeout_then_same(call, [codes, scales], monkeypatch, certain=not hadamard)
 
 
 def _attention(bits, B, T, n_rep=4):
