@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(SL * kAD) attn_combine_kernel(AttnArgs a) {
 // blocks per row, 7.5 of them unpacking; 87 in the kernel it replaced, whose value sums ran on CUDA
 // cores; with the queries as the 16-row operand instead, twice the MMAs for four queries, 308 us
 // against 298). One layer, 64 sequences x 8 heads x 16,384 tokens, 4 bits, 4 queries a head: whole
-// call 1043 -> 268 us (stream kernel 242 us, 5.0 TB/s, 73 % of measured HBM); one 32,767-token
+// call 1043 -> 268 us (stream kernel 243 us, 5.0 TB/s, 73 % of measured HBM); one 32,767-token
 // sequence at 8 bits 280 -> 42 us.
 // ------------------------------------------------------------------------------------
 constexpr int kSThreads = 128;

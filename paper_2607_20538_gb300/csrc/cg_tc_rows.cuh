@@ -407,10 +407,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_rows_encode_kernel(const __gri
         // 8-bit codes nearly always have mu >= 1e-4: their usual loop tracks the distances too
         constexpr bool kTrack = (TILE || BITS == 8) && !MASKS;
         // Search, several blocks a row: one call site of the exact round for full and last lists (the
-        // epilogue's code size sets its instruction fetch; 8B-shaped cache 594 -> 552 us; one block a row
-        // and tiles measured 1 to 3 % faster with two). Four blocks: the exact extremes of one block at a
-        // time in registers, no spills (27B-shaped cache at 6 bits 4360 -> 3925 us)
-        constexpr bool kOneSite = NBK > 1 && !TILE;
+        // epilogue's code size sets its instruction fetch; 8B-shaped cache 594 -> 552 us, tiles of 32 and 64
+        // channels 2 to 11 %; one block a row measured 1 to 3 % faster with two). Four blocks: the exact
+        // extremes of one block at a time in registers, no spills (27B-shaped cache at 6 bits 4360 -> 3925 us)
+        constexpr bool kOneSite = NBK > 1;
         constexpr bool kInPlace = NBK == 4 && !TILE && !MASKS;
         constexpr int kJobSlots = NBK == 2 ? 4 : 2;  // values per lane and memory round trip
         constexpr int kListCap = (32 + kJobCap) / 2;  // MASKS: jobs and results share the warp's buffer
